@@ -84,7 +84,8 @@ typedef struct cm_options {
     int32_t block_slots;    /* grid mode, insert: a vertex with at least this many slots (below hub_slots)
                                is scanned by a whole block instead of one warp (4096) */
     int32_t block_slots_delete; /* the same for delete calls (1024) */
-    int32_t task_claim;     /* grid mode: most search tasks a warp claims at once (1..8, default 1) */
+    int32_t task_claim;     /* grid mode: multiple of its fair share of the waiting search tasks that a warp
+                               claims at once (1..8, default 1) */
     int32_t select_order;   /* order of the greedy superior-edge-set selection (Section IV,
                                Definition 6 and Algorithm 2): CM_SELECT_HASH (default) ranks an edge
                                by fmix64 of its canonical key (lo << 32 | hi), a fixed pseudo-random
@@ -335,7 +336,7 @@ typedef struct cm_step_config {
     int32_t hub_slots;         /* frontier granularity: grid-wide chunked scans from this many slots (0 = 1024, -1 never) */
     int32_t blocks_per_sm;     /* block shape of the grid-mode launch: resident 512-thread blocks per SM (0 = max) */
     int32_t block_slots;       /* frontier granularity: block-wide scans from this many slots, insert phase (0 = 4096) */
-    int32_t task_claim;        /* most search tasks a warp claims at once (0 = 1) */
+    int32_t task_claim;        /* multiple of its fair share of the waiting search tasks that a warp claims (0 = 1) */
     int32_t reserved;
 } cm_step_config;
 

@@ -70,6 +70,12 @@ struct cm_graph {
     HubItem* HQ = nullptr;
     unsigned long long* TQ = nullptr;   // grid-mode task queue (TASK_EMPTY = all ones when free)
     unsigned long long tq_size = 0;
+    // candidate records of the grid-mode search (cm_search.cuh): per vertex
+    // a stamped position in the arena
+    unsigned long long* rec = nullptr;
+    size_t rec_size = 0;
+    int32_t* arena = nullptr;
+    unsigned long long arena_quads = 0;
     int32_t hub_len = 1024;
     int32_t block_len = 4096, block_len_del = 1024;
     int32_t claim_max = 1;
@@ -272,7 +278,11 @@ static int ensure_index(cm_graph* h, long long adding) {
 // frontier and being evicted once per iteration, plus the chunk tasks of
 // high-degree lists (three passes per list, at least 128 slots per hub) and
 // the claims warps make past the tail.
+static int ensure_records(cm_graph* h);
+
 static int ensure_tasks(cm_graph* h) {
+    int rc = ensure_records(h);
+    if (rc) return rc;
     const unsigned long long need =
         pow2_at_least(2ull * (unsigned long long)h->ncap + (unsigned long long)h->g.adj_cap / 32 + (1ull << 18));
     if (need <= h->tq_size) return CM_OK;
@@ -285,6 +295,35 @@ static int ensure_tasks(cm_graph* h) {
     }
     h->TQ = q;
     h->tq_size = need;
+    return CM_OK;
+}
+
+// Candidate records of the search: a word per vertex, and an arena of a
+// quarter of the adjacency pool for one iteration's records (a search that
+// fills it scans the lists of the vertices left out again).
+static int ensure_records(cm_graph* h) {
+    if (h->rec_size < (size_t)h->ncap) {
+        unsigned long long* q = (unsigned long long*)dalloc(h, (size_t)h->ncap * 8);
+        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the candidate records");
+        CK(h, cudaMemsetAsync(q, 0, (size_t)h->ncap * 8, h->stream));   // stamp 0 names no iteration
+        if (h->rec) {
+            CK(h, cudaStreamSynchronize(h->stream));
+            dfree(h, h->rec, h->rec_size * 8);
+        }
+        h->rec = q;
+        h->rec_size = (size_t)h->ncap;
+    }
+    const unsigned long long quads = (unsigned long long)h->g.adj_cap / 16 + 1024;
+    if (h->arena_quads < quads) {
+        int32_t* q = (int32_t*)dalloc(h, (size_t)quads * 16);
+        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the candidate arena");
+        if (h->arena) {
+            CK(h, cudaStreamSynchronize(h->stream));
+            dfree(h, h->arena, (size_t)h->arena_quads * 16);
+        }
+        h->arena = q;
+        h->arena_quads = quads;
+    }
     return CM_OK;
 }
 
@@ -389,6 +428,8 @@ static void free_all(cm_graph* h) {
     dfree(h, h->OVL, qn * 4);
     dfree(h, h->HQ, kHubRing * sizeof(HubItem));
     dfree(h, h->TQ, h->tq_size * 8);
+    dfree(h, h->rec, h->rec_size * 8);
+    dfree(h, h->arena, (size_t)h->arena_quads * 16);
     dfree(h, h->dbatch, (size_t)h->batch_cap * 8);
     dfree(h, h->bset, h->bset_size * sizeof(BSet));
     dfree(h, h->R0, (size_t)h->rcap * sizeof(REdge));
@@ -694,6 +735,13 @@ static MaintainParams handle_params(const cm_graph* h, int op) {
     p.HQ = h->HQ;
     p.TQ = h->TQ;
     p.tqmask = h->tq_size - 1;
+    p.rec = h->rec;
+    p.arena = h->arena;
+    p.arena_quads = h->arena_quads;
+    {   // a slab for every warp of the largest grid takes a quarter of the arena at most
+        const unsigned long long per = h->arena_quads / (4ull * (unsigned long long)h->num_sms * 32ull);
+        p.slab_quads = (uint32_t)(per < 32 ? 32 : per > 1024 ? 1024 : per);
+    }
     p.hub_len = h->hub_len;
     p.block_len = op == CM_OP_INSERT ? h->block_len : h->block_len_del;
     p.claim_max = h->claim_max;
@@ -781,6 +829,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
             CK(h, cudaMemsetAsync(g.chg, 0, (size_t)h->n * 4, h->stream));
             CK(h, cudaMemsetAsync(g.taken, 0, (size_t)h->n * 4, h->stream));
             CK(h, cudaMemsetAsync(g.hw, 0, (size_t)h->n * sizeof(unsigned long long), h->stream));
+            CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, h->stream));
             h->epoch = 1;
         }
         MaintainParams p = handle_params(h, op);
@@ -1321,6 +1370,9 @@ struct StepSig {   // everything a captured step bakes in
     unsigned long long qmask;
     unsigned long long* TQ;
     unsigned long long tq_size;
+    unsigned long long* rec;
+    int32_t* arena;
+    unsigned long long arena_quads;
     cudaStream_t stream;
     cm_step_config cfg;
 };
@@ -1377,6 +1429,9 @@ static StepSig step_signature(const cm_step* s) {
     z.qmask = h->qmask;
     z.TQ = h->TQ;
     z.tq_size = h->tq_size;
+    z.rec = h->rec;
+    z.arena = h->arena;
+    z.arena_quads = h->arena_quads;
     z.stream = h->stream;
     z.cfg = s->cfg;
     return z;
@@ -1653,6 +1708,7 @@ static int step_prepare(cm_step* s, long long kins) {
         CK(h, cudaMemsetAsync(g.chg, 0, (size_t)h->n * 4, h->stream));
         CK(h, cudaMemsetAsync(g.taken, 0, (size_t)h->n * 4, h->stream));
         CK(h, cudaMemsetAsync(g.hw, 0, (size_t)h->n * sizeof(unsigned long long), h->stream));
+        CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, h->stream));
         h->epoch = 1;
     }
     *s->hEpoch = h->epoch;
@@ -1839,6 +1895,7 @@ static int snap_copy(cm_graph* h, Snapshot& z, bool save) {
         h->idx_tomb = z.idx_tomb;
         h->epoch = z.epoch;
         h->n = z.n;
+        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, st));   // the stamps run again from z.epoch
     }
     return CM_OK;
 }

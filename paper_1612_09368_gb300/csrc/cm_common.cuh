@@ -90,23 +90,29 @@ struct Resume {
 constexpr int kTails = 4;
 
 // A vertex whose adjacency is scanned by all warps of a grid-mode launch,
-// in chunk tasks of kChunk slots (32 bytes; a ring of kHubRing per handle).
+// in chunk tasks of kChunk slots (64 bytes; a ring of kHubRing per handle).
 // kind: HUB_FRONT (insert frontier: chunks sum CSD, the last one decides),
 // HUB_EVICT_INS / HUB_EVICT_DEL (eviction scans), HUB_EXPAND (visit the
 // frontier neighbours of a hub whose support stayed above k).
 // HUB_FRONT_SPEC: as HUB_FRONT, but each chunk also visits its candidates
-// at once (speculative expansion, see process_frontier), so no HUB_EXPAND
-// round follows.
-enum { HUB_FRONT = 0, HUB_EVICT_INS = 1, HUB_EVICT_DEL = 2, HUB_EXPAND = 3, HUB_FRONT_SPEC = 4 };
+// at once (see expand_early) and records them, so no HUB_EXPAND round
+// follows.  HUB_EVICT_REC: eviction of the recorded candidates (off and len
+// are those of the record).
+enum {
+    HUB_FRONT = 0, HUB_EVICT_INS = 1, HUB_EVICT_DEL = 2, HUB_EXPAND = 3, HUB_FRONT_SPEC = 4, HUB_EVICT_REC = 5
+};
 struct __align__(16) HubItem {
     long long off;                 // adjacency offset
     int32_t v, kind, k, len;
     int32_t nch;                   // chunks
     int32_t acc;                   // partial-sum accumulator (HUB_FRONT)
     uint32_t done;                 // chunks finished
+    int32_t rcur;                  // recorded candidates so far
+    unsigned long long rquad;      // their record's first arena quad
+    int32_t rcap;                  // ... and room (0: none)
     int32_t pad;
 };
-constexpr int kChunk = 512;                 // slots per chunk: four 4-wide passes of one warp
+constexpr int kChunk = 512;                 // slots per chunk: one scan step of a warp
 constexpr unsigned long long kHubRing = 1ull << 20;
 constexpr unsigned long long kHubRingSafe = kHubRing - 4096;   // items in flight stay below this
 
@@ -142,6 +148,7 @@ struct __align__(128) Ctl {
     alignas(128) unsigned long long task_done;  // tasks finished
     alignas(128) unsigned long long hub_created;    // hub items of the current search
     unsigned long long hub_finished;
+    alignas(128) unsigned long long rec_top;    // next free quad of the candidate arena
     alignas(128) Resume rs;
 };
 

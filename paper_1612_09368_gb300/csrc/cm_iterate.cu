@@ -25,7 +25,7 @@
 //   insert:  positive and negative search of Algorithms 3-4, run as
 //            breadth-first waves in which both progress together (single-
 //            block mode) or as a task queue without level barriers (grid
-//            mode, below async_search: the order of processing does not
+//            mode, cm_search.cuh: the order of processing does not
 //            change the result).  The
 //            constrained endpoints are the first frontier.  Processing a
 //            frontier vertex v adds CSD(v) (Definition 8) to its support
@@ -61,13 +61,14 @@
 // and then processed by the whole block of the warp that fetched it.
 #include "cm_common.cuh"
 #include "cm_launch.h"
+#include "cm_search.cuh"
 #include "cm_vertex.cuh"
 
 namespace cm {
 
 constexpr int kBlockThreads = 512;    // single-block mode
 constexpr int kGridThreads = 512;     // grid mode, per block
-static_assert(kGridThreads / 32 == kGridWarps, "one kept-task slot per grid-mode warp");
+static_assert(kGridThreads / 32 == kGridWarps, "one search buffer per grid-mode warp");
 constexpr int kMaxBig = 64;
 constexpr int kBlockLenSingle = 256;   // single-block mode: the block scans lists from this size
 
@@ -154,259 +155,6 @@ __device__ __forceinline__ long long wave_slots(const DevGraph& g, const int32_t
     const long long total = s_sum;
     __syncthreads();
     return total;
-}
-
-// ---------------------------------------------------------------- grid-mode task queue
-// In grid mode the search of an iteration (insert: positive search and
-// evictions; delete: evictions) runs without level barriers.  Every vertex
-// that enters the frontier or is evicted also becomes a task in a queue
-// (push_vertex), and warps claim tasks one at a time until the queue is
-// quiescent: every task pushed has finished.  The proof of the interleaved
-// search does not depend on the order in which vertices are processed, so
-// the waves of the single-block mode and this order reach the same cores.
-//
-// A vertex with at least P.hub_len slots becomes a hub item instead, whose
-// list is split into kChunk-slot chunk tasks that any warp may take:
-//   HUB_FRONT: each chunk adds its share of CSD to the item; the warp that
-//     finishes the last chunk adds the sum to the support word at once
-//     (setting the processed flag, as a whole-list scan would) and either
-//     queues an expansion item (support > k) or evicts the vertex;
-//   HUB_EXPAND: each chunk visits its share of the core-k neighbours;
-//   HUB_EVICT_INS / HUB_EVICT_DEL: each chunk evicts its share; the last one
-//     lowers the core (delete) and counts the vertex.
-// The support word tolerates the delay: decrements from evicted neighbours
-// land before or after the CSD sum in any order, and a processed hub whose
-// count later falls to k is evicted by the decrement that does it.
-
-// Creates a hub item and its chunk tasks (warp-collective); false if the
-// item ring is full (the caller then scans the list itself).
-__device__ __forceinline__ bool make_hub(Ctl* C, const MaintainParams& P, int v, int kind, int k, long long off,
-                                         int len) {
-    const int lane = lane_id();
-    const int nch = (len + kChunk - 1) / kChunk;
-    unsigned long long idx = 0, tb = 0;
-    int ok = 0;
-    if (lane == 0) {
-        if (vload64(&C->hub_created) - vload64(&C->hub_finished) < kHubRingSafe) {
-            idx = atomicAdd(&C->hub_created, 1ull);
-            HubItem* it = &P.HQ[idx & (kHubRing - 1)];
-            it->off = off;
-            it->v = v;
-            it->kind = kind;
-            it->k = k;
-            it->len = len;
-            it->nch = nch;
-            it->acc = 0;
-            it->done = 0u;
-            __threadfence();   // the item before its tasks
-            tb = atomicAdd(&C->task_tail, (unsigned long long)nch);
-            ok = 1;
-        }
-    }
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (!ok) return false;
-    idx = __shfl_sync(0xffffffffu, idx, 0);
-    tb = __shfl_sync(0xffffffffu, tb, 0);
-    if (!task_room(C, P, tb, (unsigned long long)nch)) return true;   // error recorded; the search stops
-    const unsigned long long base = ((idx & (kHubRing - 1)) << kTaskChunkBits);
-    for (int j = lane; j < nch; j += 32)
-        vstore64(&P.TQ[(tb + j) & P.tqmask], mk_task(T_CHUNK, base | (unsigned long long)j));
-    return true;
-}
-
-__device__ __forceinline__ int vload32i(const int* p) { return *(const volatile int*)p; }
-
-// One chunk task (warp-collective).
-__device__ __forceinline__ void run_chunk(const DevGraph& g, Ctl* C, const MaintainParams& P, uint32_t e,
-                                          LocalStats& ls, unsigned long long payload) {
-    using WG = WarpGroup;
-    const int lane = lane_id();
-    HubItem* it = &P.HQ[payload >> kTaskChunkBits];
-    const int ci = (int)(payload & ((1ull << kTaskChunkBits) - 1));
-    // the item was written by another SM: read it from L2
-    const int v = vload32i(&it->v), kind = vload32i(&it->kind), k = vload32i(&it->k);
-    const int len = vload32i(&it->len), nch = vload32i(&it->nch);
-    const long long off = (long long)vload64((const unsigned long long*)&it->off);
-    const int s0 = ci * kChunk, s1 = min(s0 + kChunk, len);
-    if (kind == HUB_FRONT || kind == HUB_FRONT_SPEC) {
-        const int part = WG::sum(kind == HUB_FRONT_SPEC ? csd_expand_range<WG, true>(g, C, P, k, off, s0, s1, e)
-                                                        : csd_part<WG>(g, k, off, s0, s1));
-        int decide = 0;   // 1 expand, 2 evict
-        if (lane == 0) {
-            atomicAdd(&it->acc, part);
-            __threadfence();
-            if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
-                __threadfence();
-                const int acc = atomicAdd(&it->acc, 0);
-                uint32_t of;
-                int32_t oc;
-                add_word(g, C, v, e, acc, kProcessed, of, oc);
-                ls.vis++;
-                ls.visl += len;
-                decide = oc + acc > k ? 1 : 2;
-                atomicAdd(&C->hub_finished, 1ull);
-            }
-        }
-        decide = __shfl_sync(0xffffffffu, decide, 0);
-        if (decide == 1 && kind == HUB_FRONT && !make_hub(C, P, v, HUB_EXPAND, k, off, len))
-            expand_range<WG, true>(g, C, P, k, off, 0, len, e);
-        if (decide == 2) push_vertex<true>(C, P, lane == 0, v, 1, true);
-        return;
-    }
-    if (kind == HUB_EXPAND) expand_range<WG, true>(g, C, P, k, off, s0, s1, e);
-    else if (kind == HUB_EVICT_INS) evict_ins_range<WG, true>(g, C, P, k, off, s0, s1, e);
-    else evict_del_range<WG, true>(g, C, P, k, off, s0, s1, e);
-    __syncwarp();
-    if (lane == 0) {
-        __threadfence();
-        if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
-            if (kind == HUB_EVICT_DEL) {
-                g.hc[v].x = k - 1;
-                g.kc[v] = key_of(k - 1, 0);   // the SD fix-up of the next claim phase sets its bit
-            }
-            if (kind != HUB_EXPAND) {
-                ls.ev++;
-                ls.evl += len;
-            }
-            atomicAdd(&C->hub_finished, 1ull);
-        }
-    }
-}
-
-// Search (iteration number) whose queue the block's poller found quiescent.
-__shared__ volatile uint32_t s_quiet;
-
-// Drains the task queue (every warp of the grid).  Returns false on error.
-// A warp claims up to P.claim_max consecutive slots with one atomic: it
-// doubles its claim while its slots are ready at once and drops back to one
-// slot after a wait.  One slot at a time balances best when tasks are large
-// (a warp holding a run of large tasks leaves others idle); several save
-// head-counter traffic when tasks are tiny (the many-graph workload), so the
-// limit is a schedule knob.  Finished tasks are reported in batches, always
-// before the warp waits on an empty slot (so a waiting warp never holds back
-// the quiescence test).  Inlined into the kernel: as a separate function it
-// took the graph and the parameters by reference, which put both in local
-// memory and made every pointer it used a local load (measured 8-15% slower
-// per call, although the inlined kernel spills more registers).
-__device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const MaintainParams& P, uint32_t e,
-                                          LocalStats& ls) {
-    using WG = WarpGroup;
-    const int lane = lane_id();
-    const unsigned long long t_start = gtimer();
-    unsigned long long idx = 0, ndone = 0;
-    int left = 0, claim = 1;
-    bool waited = false;
-    const int cmax = P.claim_max > 1 ? P.claim_max : 1;
-    // one warp per block tests quiescence and tells the others through
-    // shared memory: a test reads two hot counters, and thousands of
-    // waiting warps reading them would slow the claims and pushes that
-    // share those counters' L2 slices
-    const bool poller = threadIdx.x < 32;
-    if (lane == 0) kept_task() = TASK_EMPTY;
-    __syncwarp();
-    for (;;) {
-        unsigned long long t = kept_task();
-        int quit = 0;
-        const bool own = t != TASK_EMPTY;   // the task this warp kept from its last one
-        __syncwarp();
-        if (own) {
-            if (lane == 0) kept_task() = TASK_EMPTY;
-        } else if (lane == 0) {
-            if (left == 0) {
-                claim = waited ? 1 : min(2 * claim, cmax);
-                waited = false;
-                idx = atomicAdd(&C->task_head, (unsigned long long)claim);
-                left = claim;
-            }
-            unsigned long long* slot = &P.TQ[idx & P.tqmask];
-            unsigned int nap = 32;
-            for (unsigned int spins = 0;; spins++) {
-                t = vload64(slot);
-                if (t != TASK_EMPTY) {
-                    vstore64(slot, TASK_EMPTY);   // free for the next search
-                    break;
-                }
-                waited = true;
-                if (ndone) {   // report before waiting
-                    __threadfence();
-                    atomicAdd(&C->task_done, ndone);
-                    ndone = 0;
-                }
-                if (poller) {
-                    // quiescent: every task pushed has finished (done read first)
-                    const unsigned long long d = ld_acquire64(&C->task_done);   // read before the tail
-                    if (d == vload64(&C->task_tail) || vload32(&C->error)) {
-                        s_quiet = e;
-                        quit = 1;
-                        break;
-                    }
-                } else if (s_quiet == e) {
-                    quit = 1;
-                    break;
-                }
-                if ((spins & 3u) == 0 && gtimer() - t_start > P.limit_ns) {
-                    atomicCAS(&C->error, 0, E_BARRIER_TIMEOUT);
-                    quit = 1;
-                    break;
-                }
-                __nanosleep(nap);
-                if (nap < 512) nap <<= 1;
-            }
-            idx++;
-            left--;
-        }
-        if (__shfl_sync(0xffffffffu, quit, 0)) break;
-        t = __shfl_sync(0xffffffffu, t, 0);
-        __syncwarp();
-        // acquire: the task's vertex data as its producers left it (measured
-        // necessary: without it, warps running several claimed tasks in a
-        // row reached wrong cores on small delete batches)
-        __threadfence();
-        const int type = (int)(t >> 62);
-        const unsigned long long payload = t & ((1ull << 62) - 1);
-        if (type == T_CHUNK) {
-            run_chunk(g, C, P, e, ls, payload);
-        } else {
-            const int v = (int)payload;
-            const VInfo vi = load_vinfo(g, v);
-            const bool hub = P.hub_len > 0 && vi.len >= P.hub_len;
-            if (type == T_FRONT) {
-                if (!hub || !make_hub(C, P, v, expand_early(P, vi.h.y, vi.h.x) ? HUB_FRONT_SPEC : HUB_FRONT, vi.h.x,
-                                      vi.o, vi.len))
-                    process_frontier<WG, true>(g, C, P, v, vi, e, ls);
-            } else if (P.op == 0) {
-                if (!hub || !make_hub(C, P, v, HUB_EVICT_INS, vi.h.x, vi.o, vi.len))
-                    evict_insert_vertex<WG, true>(g, C, P, vi, e, ls);
-            } else {
-                if (!hub || !make_hub(C, P, v, HUB_EVICT_DEL, vi.h.x, vi.o, vi.len))
-                    evict_delete_vertex<WG, true>(g, C, P, v, vi, e, ls);
-            }
-        }
-        __syncwarp();
-        // this task's pushes precede the fence of the next report; a kept
-        // task was never counted in the tail
-        if (lane == 0 && !own) ndone++;
-    }
-    return vload32(&C->error) == 0;
-}
-
-// Queues tasks for log entries [lo, hi) that are already in the log (a
-// search resumed from the single-block mode).  Every warp calls it.
-__device__ __forceinline__ void seed_tasks(Ctl* C, const MaintainParams& P, const int32_t* log, unsigned long long lo,
-                                           unsigned long long hi, int type) {
-    const int lane = lane_id();
-    const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (unsigned long long base = lo + (unsigned long long)gwarp * 32; base < hi;
-         base += (unsigned long long)nwarps * 32) {
-        const unsigned long long cnt = min(32ull, hi - base);
-        unsigned long long tb = 0;
-        if (lane == 0) tb = atomicAdd(&C->task_tail, cnt);
-        tb = __shfl_sync(0xffffffffu, tb, 0);
-        if (task_room(C, P, tb, cnt) && (unsigned long long)lane < cnt)
-            vstore64(&P.TQ[(tb + lane) & P.tqmask],
-                     mk_task(type, (unsigned long long)(uint32_t)log[(base + lane) & P.qmask]));
-    }
 }
 
 // An edge's core number k = min(core(lo), core(hi)) and its constrained
@@ -538,6 +286,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             C->task_done = 0;
             C->hub_created = 0;
             C->hub_finished = 0;
+            C->rec_top = 0;
         }
     };
     LocalStats ls;
@@ -695,7 +444,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
 
         if (P.op == 0) {
             // -------------------------------------------- SEARCH (insert): frontier + evictions
-            if (MODE == 0) {
+            if constexpr (MODE == 0) {
                 if (resumed) {   // the single-block mode began this search
                     reset_tasks();
                     if (!(ok = sync(PH_APPLY))) break;
@@ -704,7 +453,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     if (!(ok = sync(PH_APPLY))) break;
                 }
                 waves++;
-                ok = async_search(g, C, P, e, ls);
+                ok = async_search<false>(g, C, P, e, ls);
                 if (!(ok = sync(PH_DISCOVER) && ok)) break;
                 fhi = vload64(&C->stail[0]);
                 ehi = vload64(&C->stail[1]);
@@ -719,10 +468,10 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     }
                     waves++;
                     for_each_vertex<MODE>(g, P, &C->pc[2], P.VQ, qm, flo, fhi, [&](int v, auto grp) {
-                        process_frontier<decltype(grp), false>(g, C, P, v, load_vinfo(g, v), e, ls);
+                        process_frontier<decltype(grp)>(g, C, P, v, load_vinfo(g, v), e, ls);
                     });
                     for_each_vertex<MODE>(g, P, &C->pc[3], P.EQ, qm, elo, ehi, [&](int v, auto grp) {
-                        evict_insert_vertex<decltype(grp), false>(g, C, P, load_vinfo(g, v), e, ls);
+                        evict_insert_vertex<decltype(grp)>(g, C, P, load_vinfo(g, v), e, ls);
                     });
                     if (!(ok = sync(PH_DISCOVER))) break;
                     flo = fhi;
@@ -759,7 +508,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             fx_hi = cq_t;
         } else {
             // -------------------------------------------- EVICT (delete); evicted vertices drop by one
-            if (MODE == 0) {
+            if constexpr (MODE == 0) {
                 if (resumed) {
                     reset_tasks();
                     if (!(ok = sync(PH_APPLY))) break;
@@ -767,7 +516,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     if (!(ok = sync(PH_APPLY))) break;
                 }
                 waves++;
-                ok = async_search(g, C, P, e, ls);
+                ok = async_search<true>(g, C, P, e, ls);
                 if (!(ok = sync(PH_EVICT) && ok)) break;
                 ehi = vload64(&C->stail[1]);
             } else {
@@ -779,7 +528,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     }
                     waves++;
                     for_each_vertex<MODE>(g, P, &C->pc[2], P.EQ, qm, elo, ehi, [&](int v, auto grp) {
-                        evict_delete_vertex<decltype(grp), false>(g, C, P, v, load_vinfo(g, v), e, ls);
+                        evict_delete_vertex<decltype(grp)>(g, C, P, v, load_vinfo(g, v), e, ls);
                     });
                     if (!(ok = sync(PH_EVICT))) break;
                     elo = ehi;
@@ -824,17 +573,14 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         ok = sync(PH_FIXUP);
     }
     // statistics: one atomic per warp
-    if (lane == 0) {
-        if (ls.vis) atomicAdd(&C->st[ST_VISITED], (unsigned long long)ls.vis);
-        if (ls.visl) atomicAdd(&C->st[ST_VISSLOTS], (unsigned long long)ls.visl);
-        if (ls.ev) atomicAdd(&C->st[ST_EVICTED], (unsigned long long)ls.ev);
-        if (ls.evl) atomicAdd(&C->st[ST_EVSLOTS], (unsigned long long)ls.evl);
-        if (ls.ch) atomicAdd(&C->st[ST_CHANGED], (unsigned long long)ls.ch);
-        if (ls.chl) atomicAdd(&C->st[ST_CHSLOTS], (unsigned long long)ls.chl);
+    const uint32_t mine[7] = {ls.vis, ls.visl, ls.ev, ls.evl, ls.ch, ls.chl, ls.sel};
+    const int slot[7] = {ST_VISITED, ST_VISSLOTS, ST_EVICTED, ST_EVSLOTS, ST_CHANGED, ST_CHSLOTS, ST_SELECTED};
+#pragma unroll
+    for (int i = 0; i < 7; i++) {
+        unsigned long long t = mine[i];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0 && t) atomicAdd(&C->st[slot[i]], t);
     }
-    long long sel = ls.sel;
-    for (int o = 16; o > 0; o >>= 1) sel += __shfl_xor_sync(0xffffffffu, sel, o);
-    if (lane == 0 && sel) atomicAdd(&C->st[ST_SELECTED], (unsigned long long)sel);
     if (leader) {
         C->st[ST_ITERS] += (unsigned long long)iters;
         if (MODE == 0) C->st[ST_GRID_ITERS] += (unsigned long long)iters;
@@ -871,9 +617,16 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
     if (MODE == 1) loop_control(P, C);   // thread 0 is the leader: its writes above come first
 }
 
+// The search's buffers exceed the default 48 KB of shared memory per block.
+static cudaError_t allow_search_smem() {
+    return cudaFuncSetAttribute(maintain_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSearchSmem);
+}
+
 int maintain_blocks_per_sm(int threads) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, maintain_kernel<0>, threads, 0) != cudaSuccess) return 0;
+    if (allow_search_smem() != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, maintain_kernel<0>, threads, kSearchSmem) != cudaSuccess)
+        return 0;
     return nb;
 }
 
@@ -883,7 +636,7 @@ cudaError_t launch_maintain(const MaintainParams& p, int blocks, int threads, cu
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = kSearchSmem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;

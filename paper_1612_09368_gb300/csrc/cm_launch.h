@@ -37,9 +37,13 @@ struct MaintainParams {
     HubItem* HQ;              // hub items of the current search (ring of kHubRing)
     unsigned long long* TQ;   // grid-mode task queue (ring, TASK_EMPTY when free)
     unsigned long long tqmask;
+    unsigned long long* rec;  // per vertex: where its candidates are recorded in `arena` (stamped, see cm_search.cuh)
+    int32_t* arena;
+    unsigned long long arena_quads;
+    uint32_t slab_quads;      // arena quads a warp takes at a time
     int32_t hub_len;          // grid mode: vertices with at least this many slots are scanned grid-wide
     int32_t block_len;        // vertices with at least this many slots are scanned by a whole block
-    int32_t claim_max;        // grid-mode task queue: most slots a warp claims at once
+    int32_t claim_max;        // grid-mode task queue: multiple of its fair share of the backlog a warp claims
     int32_t sel_key;          // selection order: 0 fmix64 of the canonical key, 1 the key itself
     int32_t sel_rounds;       // claim rounds per iteration (0 = until the set is maximal)
     int32_t use_cond;         // inside a captured step: the single-block kernel drives the loop node

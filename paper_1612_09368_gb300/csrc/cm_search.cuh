@@ -1,0 +1,973 @@
+// cm_search.cuh -- grid mode: the search of one iteration as a task queue
+// (included by cm_iterate.cu only).
+//
+// In grid mode the search of an iteration (insert: positive search and
+// evictions; delete: evictions) runs without level barriers.  Every vertex
+// that enters the frontier or is evicted also becomes a task in a queue, and
+// warps claim tasks until the queue is quiescent: every task pushed has
+// finished.  The proof of the interleaved search does not depend on the
+// order in which vertices are processed, so the waves of the single-block
+// mode and this order reach the same cores.
+//
+// What bounds it: not bytes but dependent round trips.  A list step is a
+// chain list words -> the neighbours' keys -> the candidates' per-iteration
+// words -> their atomics -> the queue push, each about a microsecond away,
+// so the time is trips x steps, and the layout below puts as many slots as
+// registers allow behind each trip:
+//
+//   * a scan step is a window of 512 slots (16 per lane): four 16-byte list
+//     loads per lane, then 16 key gathers, all in flight together.  The
+//     slots that matter (candidates: core k, and for an insertion SD > k)
+//     are few; they are compacted into a per-warp shared buffer, and their
+//     words and atomics are then handled 128 at a time, every lane busy.
+//   * tasks are taken 32 at a time, one per lane.  The lists of those with
+//     at most 128 slots are walked together, quad by quad (a quad is four
+//     slots, one 16-byte load), up to 128 quads a window: lane l of a
+//     window's load takes quad l whoever owns it.  (With one warp per vertex
+//     a vertex of 9 slots used three lanes of 32 and cost a queue hand-off.)
+//   * a frontier vertex whose support stays at or below k is evicted by the
+//     task that found it out, from the candidates it still holds.
+//   * a longer list whose vertex survives leaves its candidates behind (an
+//     arena in device memory): if the vertex is evicted later, its eviction
+//     reads those few ids instead of the whole list and its keys.
+//
+// Measured search time (GB300, one warp per vertex and 128-slot steps -> this
+// layout): Erdos-Renyi, 2*10^6 vertices of degree 8, 10^4 uniform inserts 6.5
+// -> 1.9 ms; 64 Barabasi-Albert graphs (57 iterations) 27 -> 13 ms; R-MAT
+// scale 24, 10^3 degree-proportional inserts (4*10^5 vertices visited,
+// 3.8*10^8 slots) 7.5 -> 5.0 ms, of which the key gathers alone are 1.3 ms
+// at the 300 G gathers/s (one lane per clock and SM) that a kernel doing
+// nothing else reaches.
+//
+// A vertex with at least P.hub_len slots becomes a hub item instead, whose
+// list is split into kChunk-slot chunk tasks that any warp may take:
+//   HUB_FRONT / HUB_FRONT_SPEC: each chunk adds its share of CSD to the
+//     item; the warp that finishes the last chunk adds the sum to the
+//     support word at once (setting the processed flag, as a whole-list
+//     scan would) and either queues an expansion item (support > k; the
+//     SPEC chunks have visited their candidates already) or evicts the
+//     vertex;
+//   HUB_EXPAND: each chunk visits its share of the core-k neighbours;
+//   HUB_EVICT_INS / HUB_EVICT_DEL / HUB_EVICT_REC: each chunk evicts its
+//     share (REC: of the recorded candidates); the last one lowers the core
+//     (delete) and counts the vertex.
+// The support word tolerates the delay: decrements from evicted neighbours
+// land before or after the CSD sum in any order, and a processed hub whose
+// count later falls to k is evicted by the decrement that does it.
+#pragma once
+#include "cm_common.cuh"
+#include "cm_launch.h"
+#include "cm_vertex.cuh"
+
+namespace cm {
+
+constexpr int kGridWarps = 16;    // warps per grid-mode block
+constexpr int kWindow = 512;      // slots of a scan step
+constexpr int kCand = 1024;       // candidates a warp holds: every list below the default hub_len fits
+constexpr int kShort = 128;       // lists up to this many slots are walked together
+
+// Per-warp scratch of the search (dynamic shared memory).
+struct WarpBuf {
+    int32_t id[kCand];                // candidates
+    unsigned long long kept[32];      // tasks the warp keeps for itself
+    int32_t csd[32];                  // CSD of the tasks walked together
+    uint8_t own[kWindow];             // their candidates' tasks (lane numbers)
+};
+constexpr size_t kSearchSmem = sizeof(WarpBuf) * kGridWarps;
+extern __shared__ __align__(16) unsigned char s_search[];
+
+__device__ __forceinline__ int vload32i(const int* p) { return *(const volatile int*)p; }
+
+// A vertex's record: the stamp of the iteration that wrote it (30 bits, as
+// in the per-iteration word) and the arena quad where its candidates start
+// (the first quad holds their count).  One 64-bit word, so a reader sees
+// both or neither; a stale stamp means "scan the list".
+__device__ __forceinline__ unsigned long long rec_word(unsigned long long quad, uint32_t e) {
+    return (quad << 30) | (unsigned long long)(e & 0x3FFFFFFFu);
+}
+__device__ __forceinline__ bool rec_of(unsigned long long w, uint32_t e, unsigned long long& quad) {
+    quad = w >> 30;
+    return (uint32_t)(w & 0x3FFFFFFFull) == (e & 0x3FFFFFFFu);
+}
+
+// What a warp carries through a search besides its buffer.
+struct Walker {
+    int nk;        // kept tasks
+    int klim;      // most it may keep: 1 while warps wait for tasks, 32 while the queue is long
+    int nrec;      // records made but not published: lane i < nrec holds one
+    int rec_v;
+    unsigned long long rec_q;
+    unsigned long long slab, slab_end;   // arena quads it holds
+};
+
+// ---------------------------------------------------------------- pushes
+// Appends the vertices of the lanes' bit masks (bit j: id[j]) to the logs
+// and the task queue: `fm` enter the frontier (insert), `em` are evicted.
+// One atomic per counter for the warp, issued by three lanes at once.  The
+// first few stay with the warp (W.klim): it runs them next, which saves the
+// hand-off through the queue.  A kept task is not counted in the queue's
+// tail and not reported done; the task that produced it is reported only
+// when the warp has run out of kept tasks, so quiescence still waits for it.
+// Evictions are kept first: they prune the search.  Warp-collective.
+template <int J>
+__device__ __forceinline__ void push_new(Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W, unsigned fm,
+                                         unsigned em, const int (&id)[J]) {
+    if (!__any_sync(0xffffffffu, (fm | em) != 0)) return;
+    const int lane = lane_id();
+    const unsigned mine = (unsigned)__popc(fm) | ((unsigned)__popc(em) << 16);
+    unsigned incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const unsigned tot = __shfl_sync(0xffffffffu, incl, 31);
+    const int nf = (int)(tot & 0xFFFFu), ne = (int)(tot >> 16);
+    const int kq = min(W.klim - W.nk > 0 ? W.klim - W.nk : 0, nf + ne);
+    const unsigned long long nq = (unsigned long long)(nf + ne - kq);
+    unsigned long long base = 0;
+    if (lane < 3) {
+        unsigned long long* p = lane == 0 ? &C->tail[0] : lane == 1 ? &C->tail[1] : &C->task_tail;
+        const unsigned long long n = lane == 0 ? (unsigned long long)nf : lane == 1 ? (unsigned long long)ne : nq;
+        if (n) base = atomicAdd(p, n);
+    }
+    const unsigned long long fb = __shfl_sync(0xffffffffu, base, 0);
+    const unsigned long long eb = __shfl_sync(0xffffffffu, base, 1);
+    const unsigned long long tb = __shfl_sync(0xffffffffu, base, 2);
+    const bool room = nq == 0 || task_room(C, P, tb, nq);
+    const unsigned excl = incl - mine;
+    int fr = (int)(excl & 0xFFFFu), er = (int)(excl >> 16);
+#pragma unroll
+    for (int j = 0; j < J; j++) {
+        const bool f = (fm >> j) & 1u, x = (em >> j) & 1u;
+        if (!f && !x) continue;
+        const int rank = x ? er : ne + fr;
+        if (x) P.EQ[(eb + er++) & P.qmask] = id[j];
+        else P.VQ[(fb + fr++) & P.qmask] = id[j];
+        const unsigned long long task = mk_task(x ? T_EVICT : T_FRONT, (unsigned long long)(uint32_t)id[j]);
+        if (rank < kq) B.kept[W.nk + rank] = task;
+        else if (room) vstore64(&P.TQ[(tb + (unsigned)(rank - kq)) & P.tqmask], task);
+    }
+    W.nk += kq;
+    __syncwarp();
+}
+
+// ---------------------------------------------------------------- scan of one list
+// Slots [s, min(s + 128 U, len)) of a list of a vertex at level k: adds
+// this lane's share of CSD to `part` (insert: the neighbours above k and the
+// candidates, Definition 8) and, if `store`, appends the candidates to the
+// buffer behind the nc it holds.  Returns the new count.  Lists start
+// 16-byte aligned and their capacity is a multiple of 4; they are read
+// evict-first so that L2 keeps the keys.  Warp-collective.
+template <bool DEL, int U = 4>
+__device__ __forceinline__ int scan_window(const DevGraph& g, const int32_t* list, int s, int len, int k, bool store,
+                                           WarpBuf& B, int nc, int& part) {
+    const int lane = lane_id();
+    int id[4 * U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+        const int t = s + u * 128 + lane * 4;
+        int4 a = make_int4(HOLE, HOLE, HOLE, HOLE);
+        if (t < len) a = __ldcs(reinterpret_cast<const int4*>(list + t));
+        id[4 * u] = a.x;
+        id[4 * u + 1] = t + 1 < len ? a.y : HOLE;
+        id[4 * u + 2] = t + 2 < len ? a.z : HOLE;
+        id[4 * u + 3] = t + 3 < len ? a.w : HOLE;
+    }
+    uint32_t key[4 * U];
+#pragma unroll
+    for (int i = 0; i < 4 * U; i++) key[i] = id[i] >= 0 ? g.kc[id[i]] : KEY_DEAD;
+    unsigned mask = 0;
+#pragma unroll
+    for (int i = 0; i < 4 * U; i++) {
+        if (DEL) {
+            mask |= key_core(key[i]) == k ? 1u << i : 0u;
+        } else {   // key order is (core, bit): above k or a candidate <=> key >= 2k + 1
+            part += (int)key[i] >= 2 * k + 1;
+            mask |= key[i] == (uint32_t)(2 * k + 1) ? 1u << i : 0u;
+        }
+    }
+    if (!store || !__any_sync(0xffffffffu, mask != 0)) return nc;
+    const int cnt = __popc(mask);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    int at = nc + incl - cnt;
+#pragma unroll
+    for (int i = 0; i < 4 * U; i++)
+        if ((mask >> i) & 1u) B.id[at++] = id[i];
+    nc += __shfl_sync(0xffffffffu, incl, 31);
+    __syncwarp();
+    return nc;
+}
+
+// ---------------------------------------------------------------- candidates
+// The nc buffered candidates of an insertion search, 32 J at a time: of a
+// vertex whose support exceeds its level, visit (those not visited yet enter
+// the frontier, Algorithm 3); of an evicted one, take one from the support,
+// and a processed candidate whose support falls to k leaves too (Algorithm
+// 4).  MANY: candidate i belongs to the task of lane B.own[i], with that
+// lane's level k and bit of the mask that decide() returns (set: visit);
+// otherwise all belong to one task, with level k and bit 0.  decide() runs
+// once, after the first words are requested, so the support atomics that it
+// waits for overlap them.  Warp-collective.
+template <bool MANY, int J = 4, class Decide>
+__device__ __forceinline__ void act_insert(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                           int nc, int k, uint32_t e, Decide decide) {
+    const int lane = lane_id();
+    const unsigned long long dec = 0xFFFFFFFF00000000ull;   // one off the count
+    unsigned vmask = 0;
+    for (int b0 = 0; b0 == 0 || b0 < nc; b0 += 32 * J) {
+        int id[J], kk[J], ow[J];
+        unsigned long long s[J];
+        unsigned vis = 0, go = 0, cur = 0;
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            const int i = b0 + j * 32 + lane;
+            id[j] = i < nc ? B.id[i] : -1;
+            ow[j] = MANY && i < nc ? B.own[i] : 0;
+            kk[j] = MANY ? __shfl_sync(0xffffffffu, k, ow[j]) : k;
+            s[j] = id[j] >= 0 ? __ldcg(iter_word(g, id[j])) : 0ull;
+        }
+        if (b0 == 0) vmask = decide();
+#pragma unroll
+        for (int j = 0; j < J; j++) vis |= ((vmask >> ow[j]) & 1u) << j;
+        unsigned long long r[J];
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            r[j] = 0;
+            if (id[j] < 0) continue;
+            const bool same = same_iter(wz(s[j]), e), v = (vis >> j) & 1u;
+            if (same && (v ? (wz(s[j]) & kVisited) != 0 : (wz(s[j]) & kProcessed) && ww(s[j]) <= kk[j])) continue;
+            go |= 1u << j;
+            unsigned long long* p = iter_word(g, id[j]);
+            if (!same) {
+                r[j] = atomicCAS(p, s[j], (v ? (unsigned long long)kVisited : dec) | (unsigned long long)(e << 2));
+            } else {
+                cur |= 1u << j;
+                r[j] = v ? atomicOr(p, (unsigned long long)kVisited) : atomicAdd(p, dec);
+            }
+        }
+        unsigned fm = 0, em = 0;
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            if (!((go >> j) & 1u)) continue;
+            const bool v = (vis >> j) & 1u;
+            if (!((cur >> j) & 1u)) {
+                if (r[j] == s[j]) {           // first to touch it in this iteration
+                    fm |= v ? 1u << j : 0u;
+                    continue;
+                }
+                make_current(g, C, id[j], e, r[j]);
+                r[j] = v ? atomicOr(iter_word(g, id[j]), (unsigned long long)kVisited)
+                         : atomicAdd(iter_word(g, id[j]), dec);
+            }
+            if (v) fm |= (wz(r[j]) & kVisited) == 0 ? 1u << j : 0u;
+            else em |= (wz(r[j]) & kProcessed) && ww(r[j]) == kk[j] + 1 ? 1u << j : 0u;
+        }
+        push_new<J>(C, P, B, W, fm, em, id);
+    }
+}
+
+// Recorded candidates [i0, i1) of an evicted vertex at level k.  Its own
+// expansion visited every one of them in this iteration (the record is
+// published after that), so their words carry the iteration's stamp and a
+// plain add does.  Warp-collective.
+__device__ __forceinline__ void act_recorded(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                             const int32_t* list, int i0, int i1, int k) {
+    const int lane = lane_id();
+    for (int b0 = i0; b0 < i1; b0 += 128) {
+        int id[4];
+        unsigned long long r[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int i = b0 + j * 32 + lane;
+            id[j] = i < i1 ? __ldcg(list + i) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            r[j] = id[j] >= 0 ? atomicAdd(iter_word(g, id[j]), 0xFFFFFFFF00000000ull) : 0ull;
+        unsigned em = 0;
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            em |= id[j] >= 0 && (wz(r[j]) & kProcessed) && ww(r[j]) == k + 1 ? 1u << j : 0u;
+        push_new<4>(C, P, B, W, 0u, em, id);
+    }
+}
+
+// The nc buffered candidates (core-k neighbours) of vertices evicted by a
+// deletion: each loses one support, initially its SD, and leaves when its
+// count of evicted neighbours reaches SD - k + 1 (Algorithm 7).  Evicted
+// vertices (chg == e) are skipped: their cores already dropped, so one that
+// fell from k + 1 would pass for level k.
+template <bool MANY, int J = 4>
+__device__ __forceinline__ void act_delete(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                           int nc, int k, uint32_t e) {
+    const int lane = lane_id();
+    const unsigned long long inc = 1ull << 32;
+    for (int b0 = 0; b0 < nc; b0 += 32 * J) {
+        int id[J], thr[J];
+        unsigned long long s[J];
+        uint32_t ch[J];
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            const int i = b0 + j * 32 + lane;
+            id[j] = i < nc ? B.id[i] : -1;
+            const int o = MANY && i < nc ? B.own[i] : 0;
+            const int kk = MANY ? __shfl_sync(0xffffffffu, k, o) : k;
+            s[j] = id[j] >= 0 ? __ldcg(iter_word(g, id[j])) : 0ull;
+            ch[j] = id[j] >= 0 ? __ldcg(g.chg + id[j]) : e;   // from L2: never older than the key
+            thr[j] = id[j] >= 0 ? g.hc[id[j]].y - kk + 1 : 0;
+        }
+        unsigned long long r[J];
+        unsigned go = 0;
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            r[j] = 0;
+            const bool same = same_iter(wz(s[j]), e);
+            if (ch[j] == e || thr[j] <= 0 || (same && ww(s[j]) >= thr[j])) continue;
+            go |= 1u << j;
+            r[j] = same ? atomicAdd(iter_word(g, id[j]), inc)
+                        : atomicCAS(iter_word(g, id[j]), s[j], inc | (unsigned long long)(e << 2));
+        }
+        unsigned em = 0;
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            if (!((go >> j) & 1u)) continue;
+            int oc = 0;
+            if (same_iter(wz(s[j]), e)) {
+                oc = ww(r[j]);
+            } else if (r[j] != s[j]) {   // someone touched it first: restamp if needed, then add
+                make_current(g, C, id[j], e, r[j]);
+                oc = ww(atomicAdd(iter_word(g, id[j]), inc));
+            }
+            if (oc + 1 == thr[j]) {
+                g.chg[id[j]] = e;
+                em |= 1u << j;
+            }
+        }
+        push_new<J>(C, P, B, W, 0u, em, id);
+    }
+}
+
+// ---------------------------------------------------------------- hub items
+// Creates a hub item and its chunk tasks (warp-collective); false if the
+// item ring is full (the caller then scans the list itself).  sd > 0: the
+// item also reserves arena room for sd recorded candidates.
+__device__ __forceinline__ bool make_hub(Ctl* C, const MaintainParams& P, int v, int kind, int k, long long off,
+                                         int len, int sd) {
+    const int lane = lane_id();
+    const int nch = (len + kChunk - 1) / kChunk;
+    unsigned long long idx = 0, tb = 0;
+    int ok = 0;
+    if (lane == 0) {
+        if (vload64(&C->hub_created) - vload64(&C->hub_finished) < kHubRingSafe) {
+            idx = atomicAdd(&C->hub_created, 1ull);
+            unsigned long long rb = 0;
+            int rcap = 0;
+            if (sd > 0) {
+                const unsigned long long q = 1ull + (unsigned long long)((sd + 3) >> 2);
+                rb = atomicAdd(&C->rec_top, q);
+                if (rb + q <= P.arena_quads) rcap = sd;
+            }
+            HubItem* it = &P.HQ[idx & (kHubRing - 1)];
+            it->off = off;
+            it->v = v;
+            it->kind = kind;
+            it->k = k;
+            it->len = len;
+            it->nch = nch;
+            it->acc = 0;
+            it->done = 0u;
+            it->rcur = 0;
+            it->rquad = rb;
+            it->rcap = rcap;
+            __threadfence();   // the item before its tasks
+            tb = atomicAdd(&C->task_tail, (unsigned long long)nch);
+            ok = 1;
+        }
+    }
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    if (!ok) return false;
+    idx = __shfl_sync(0xffffffffu, idx, 0);
+    tb = __shfl_sync(0xffffffffu, tb, 0);
+    if (!task_room(C, P, tb, (unsigned long long)nch)) return true;   // error recorded; the search stops
+    const unsigned long long base = ((idx & (kHubRing - 1)) << kTaskChunkBits);
+    for (int j = lane; j < nch; j += 32)
+        vstore64(&P.TQ[(tb + j) & P.tqmask], mk_task(T_CHUNK, base | (unsigned long long)j));
+    return true;
+}
+
+// One vertex pushed by the warp (an evicted hub).
+__device__ __forceinline__ void push_evicted(Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W, int v) {
+    const int id[1] = {v};
+    push_new<1>(C, P, B, W, 0u, lane_id() == 0 ? 1u : 0u, id);
+}
+
+// One chunk task (warp-collective).
+__device__ __forceinline__ void run_chunk(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                          uint32_t e, LocalStats& ls, unsigned long long payload) {
+    const int lane = lane_id();
+    HubItem* it = &P.HQ[payload >> kTaskChunkBits];
+    const int ci = (int)(payload & ((1ull << kTaskChunkBits) - 1));
+    // the item was written by another SM: read it from L2
+    const int v = vload32i(&it->v), kind = vload32i(&it->kind), k = vload32i(&it->k);
+    const int len = vload32i(&it->len), nch = vload32i(&it->nch), rcap = vload32i(&it->rcap);
+    const long long off = (long long)vload64((const unsigned long long*)&it->off);
+    const unsigned long long rquad = vload64(&it->rquad);
+    const int s0 = ci * kChunk, s1 = min(s0 + kChunk, len);
+    if (kind == HUB_FRONT || kind == HUB_FRONT_SPEC) {
+        const bool spec = kind == HUB_FRONT_SPEC;
+        int part = 0;
+        const int nc = scan_window<false>(g, g.adj + off, s0, s1, k, spec, B, 0, part);
+        part = warp_sum(part);
+        if (spec && nc > 0) {
+            int at = 0;
+            if (lane == 0 && rcap > 0) at = atomicAdd(&it->rcur, nc);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (rcap > 0 && at + nc <= rcap) {
+                int32_t* out = P.arena + 4 * rquad + 4 + at;
+                for (int i = lane; i < nc; i += 32) out[i] = B.id[i];
+            }
+            act_insert<false>(g, C, P, B, W, nc, k, e, [] { return 1u; });
+        }
+        __syncwarp();
+        int decide = 0;   // 1 expand, 2 evict
+        if (lane == 0) {
+            atomicAdd(&it->acc, part);
+            __threadfence();
+            if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
+                __threadfence();
+                const int acc = atomicAdd(&it->acc, 0);
+                const int rcur = atomicAdd(&it->rcur, 0);
+                if (rcap > 0 && rcur <= rcap) {   // the record before the flag that lets others evict v
+                    P.arena[4 * rquad] = rcur;
+                    __threadfence();
+                    vstore64(&P.rec[v], rec_word(rquad, e));
+                }
+                uint32_t of;
+                int32_t oc;
+                add_word(g, C, v, e, acc, kProcessed, of, oc);
+                ls.vis++;
+                ls.visl += len;
+                decide = oc + acc > k ? 1 : 2;
+                atomicAdd(&C->hub_finished, 1ull);
+            }
+        }
+        decide = __shfl_sync(0xffffffffu, decide, 0);
+        if (decide == 1 && !spec && !make_hub(C, P, v, HUB_EXPAND, k, off, len, 0)) {
+            for (int s = 0; s < len; s += kWindow) {
+                const int m = scan_window<false>(g, g.adj + off, s, len, k, true, B, 0, part);
+                act_insert<false>(g, C, P, B, W, m, k, e, [] { return 1u; });
+            }
+        }
+        if (decide == 2) push_evicted(C, P, B, W, v);
+        return;
+    }
+    int unused = 0;
+    if (kind == HUB_EVICT_REC) {
+        act_recorded(g, C, P, B, W, P.arena + off, s0, s1, k);
+    } else if (kind == HUB_EVICT_DEL) {
+        const int nc = scan_window<true>(g, g.adj + off, s0, s1, k, true, B, 0, unused);
+        act_delete<false>(g, C, P, B, W, nc, k, e);
+    } else {   // HUB_EXPAND visits, HUB_EVICT_INS evicts
+        const int nc = scan_window<false>(g, g.adj + off, s0, s1, k, true, B, 0, unused);
+        act_insert<false>(g, C, P, B, W, nc, k, e, [&] { return kind == HUB_EXPAND ? 1u : 0u; });
+    }
+    __syncwarp();
+    if (lane == 0) {
+        __threadfence();
+        if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
+            if (kind == HUB_EVICT_DEL) {
+                g.hc[v].x = k - 1;
+                g.kc[v] = key_of(k - 1, 0);   // the SD fix-up of the next claim phase sets its bit
+            }
+            if (kind != HUB_EXPAND) {
+                ls.ev++;
+                ls.evl += len;
+            }
+            atomicAdd(&C->hub_finished, 1ull);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- single lists
+// Adds a frontier vertex's CSD to its support and sets its processed flag;
+// returns the old word.  Whoever made it a frontier vertex stamped its word
+// with this iteration, so a plain add does.
+__device__ __forceinline__ unsigned long long add_csd(const DevGraph& g, int v, int csd) {
+    return atomicAdd(iter_word(g, v), ((unsigned long long)(uint32_t)csd << 32) + (unsigned long long)kProcessed);
+}
+
+// Arena room for n candidates and their count: the first quad, or NO_QUAD.
+// A warp takes room in slabs, so few records touch the shared counter; what
+// is left of a slab too small for a record is dropped.  Warp-uniform result.
+constexpr unsigned long long NO_QUAD = ~0ull;
+__device__ __forceinline__ unsigned long long arena_take(Ctl* C, const MaintainParams& P, Walker& W, int n) {
+    const unsigned need = 1u + (unsigned)((n + 3) >> 2);
+    if (W.slab_end - W.slab < need) {
+        const unsigned long long q = need > P.slab_quads ? need : P.slab_quads;
+        unsigned long long at = 0;
+        if (lane_id() == 0) at = atomicAdd(&C->rec_top, q);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at + q > P.arena_quads) return NO_QUAD;
+        W.slab = at;
+        W.slab_end = at + q;
+    }
+    const unsigned long long q = W.slab;
+    W.slab += need;
+    return q;
+}
+
+// A frontier vertex with more than kShort slots (Algorithm 3): support +=
+// CSD; above k it visits its candidates and leaves a record of them (W.rec_*:
+// published by publish_records), else it is evicted.  Nearly all of them
+// survive this step, so the candidates are visited while the support atomic
+// is under way (expand_early); one that fails after all then evicts from the
+// same buffer.  A list whose candidates do not fit the buffer (only without
+// hub items, or with a larger hub_len) is scanned again to act.
+__device__ __forceinline__ void long_front(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                           int v, int k, const int32_t* list, int len, uint32_t e, LocalStats& ls) {
+    const int lane = lane_id();
+    int nc = 0, part = 0;
+    bool spilled = false;
+    for (int s = 0; s < len; s += kWindow) {
+        spilled = spilled || nc + kWindow > kCand;
+        nc = scan_window<false>(g, list, s, len, k, !spilled, B, nc, part);
+    }
+    const int csd = warp_sum(part);
+    unsigned long long old = 0;
+    if (lane == 0) {
+        old = add_csd(g, v, csd);
+        ls.vis++;
+        ls.visl += len;
+    }
+    auto above = [&] { return __shfl_sync(0xffffffffu, ww(old) + csd > k ? 1u : 0u, 0); };
+    if (spilled) {
+        const unsigned up = above();
+        for (int s = 0; s < len; s += kWindow) {
+            const int m = scan_window<false>(g, list, s, len, k, true, B, 0, part);
+            act_insert<false>(g, C, P, B, W, m, k, e, [&] { return up; });
+        }
+        if (!up && lane == 0) ls.ev++;
+        return;
+    }
+    const bool early = expand_early(P);
+    if (nc > 0) {
+        const unsigned long long q = arena_take(C, P, W, nc);
+        if (q != NO_QUAD) {
+            int32_t* out = P.arena + 4 * q;
+            if (lane == 0) out[0] = nc;
+            for (int i = lane; i < nc; i += 32) out[4 + i] = B.id[i];
+        }
+        unsigned up = 1u;
+        act_insert<false>(g, C, P, B, W, nc, k, e, [&] {
+            if (!early) up = above();
+            return up;
+        });
+        if (early) {
+            up = above();
+            if (!up) act_insert<false>(g, C, P, B, W, nc, k, e, [] { return 0u; });
+        }
+        if (!up && lane == 0) ls.ev++;
+        // the record is complete, and every candidate carries the iteration's stamp
+        if (up && q != NO_QUAD) {
+            if (lane == W.nrec) {
+                W.rec_v = v;
+                W.rec_q = q;
+            }
+            W.nrec++;
+        }
+        return;
+    }
+    if (!above() && lane == 0) ls.ev++;
+}
+
+// Publishes the records a warp has made (at most one per lane), with one
+// fence for all of them.  A vertex that is evicted before its record is out
+// has its list scanned again.
+__device__ __forceinline__ void publish_records(const MaintainParams& P, Walker& W, uint32_t e) {
+    if (W.nrec == 0) return;
+    __syncwarp();
+    __threadfence();
+    if (lane_id() < W.nrec) vstore64(&P.rec[W.rec_v], rec_word(W.rec_q, e));
+    W.nrec = 0;
+}
+
+// An evicted vertex with more than kShort slots (insert: Algorithm 4; delete:
+// Algorithm 7, the vertex drops to k - 1).
+template <bool DEL>
+__device__ __forceinline__ void long_evict(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                           int v, int k, const int32_t* list, int len, uint32_t e, LocalStats& ls) {
+    int unused = 0;
+    for (int s = 0; s < len; s += kWindow) {
+        const int m = scan_window<DEL>(g, list, s, len, k, true, B, 0, unused);
+        if (DEL) act_delete<false>(g, C, P, B, W, m, k, e);
+        else act_insert<false>(g, C, P, B, W, m, k, e, [] { return 0u; });
+    }
+    if (lane_id() == 0) {
+        if (DEL) {
+            g.hc[v].x = k - 1;
+            g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
+        }
+        ls.ev++;
+        ls.evl += len;
+    }
+}
+
+// A task with at most kShort slots that is alone in its batch: one scan
+// step, and one candidate per lane where they fit (the walk of many short
+// lists takes about three times the instructions, which is what a lone task's
+// latency consists of once its words are in L2).
+template <bool DEL>
+__device__ __forceinline__ void lone_short(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                           int v, int k, const int32_t* list, int len, bool front, uint32_t e,
+                                           LocalStats& ls) {
+    const int lane = lane_id();
+    int part = 0;
+    const int nc = scan_window<DEL, 1>(g, list, 0, len, k, true, B, 0, part);
+    if constexpr (DEL) {
+        if (nc <= 32) act_delete<false, 1>(g, C, P, B, W, nc, k, e);
+        else act_delete<false, 4>(g, C, P, B, W, nc, k, e);
+        if (lane == 0) {
+            g.hc[v].x = k - 1;
+            g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
+            ls.ev++;
+            ls.evl += len;
+        }
+    } else {
+        unsigned long long old = 0;
+        int csd = 0;
+        if (front) {
+            csd = warp_sum(part);
+            if (lane == 0) {
+                old = add_csd(g, v, csd);
+                ls.vis++;
+                ls.visl += len;
+            }
+        } else if (lane == 0) {
+            ls.ev++;
+            ls.evl += len;
+        }
+        auto decide = [&] {
+            if (!front) return 0u;
+            const unsigned up = __shfl_sync(0xffffffffu, ww(old) + csd > k ? 1u : 0u, 0);
+            if (!up && lane == 0) ls.ev++;
+            return up;
+        };
+        if (nc <= 32) act_insert<false, 1>(g, C, P, B, W, nc, k, e, decide);
+        else act_insert<false, 4>(g, C, P, B, W, nc, k, e, decide);
+    }
+}
+
+// ---------------------------------------------------------------- a batch of tasks
+// Runs the tasks of the lanes with t != TASK_EMPTY (warp-collective).
+template <bool DEL>
+__device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                          uint32_t e, LocalStats& ls, unsigned long long t) {
+    const int lane = lane_id();
+    const bool have = t != TASK_EMPTY;
+    const int type = have ? (int)(t >> 62) : -1;
+    for (unsigned m = __ballot_sync(0xffffffffu, type == T_CHUNK); m; m &= m - 1) {
+        const unsigned long long payload = __shfl_sync(0xffffffffu, t, __ffs(m) - 1) & ((1ull << 62) - 1);
+        run_chunk(g, C, P, B, W, e, ls, payload);
+    }
+    const bool vert = type == T_FRONT || type == T_EVICT;
+    if (!__any_sync(0xffffffffu, vert)) return;
+    const bool front = !DEL && type == T_FRONT;
+    int v = 0, k = 0, sd = 0, len = 0;
+    long long off = 0;
+    unsigned long long rec = 0;
+    if (vert) {   // independent loads, issued together
+        v = (int)(uint32_t)t;
+        const int2 c = g.hc[v];
+        off = g.off[v];
+        len = g.end[v];
+        if (!DEL && !front) rec = ld_acquire64(&P.rec[v]);
+        k = c.x;
+        sd = c.y;
+    }
+    // lists of more than kShort slots, one after another
+    for (unsigned m = __ballot_sync(0xffffffffu, vert && len > kShort); m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const int xv = __shfl_sync(0xffffffffu, v, src), xk = __shfl_sync(0xffffffffu, k, src);
+        const int xlen = __shfl_sync(0xffffffffu, len, src);
+        const long long xoff = __shfl_sync(0xffffffffu, off, src);
+        const bool xfront = __shfl_sync(0xffffffffu, (int)front, src) != 0;
+        const bool hub = P.hub_len > 0 && xlen >= P.hub_len;
+        if (DEL) {
+            if (!hub || !make_hub(C, P, xv, HUB_EVICT_DEL, xk, xoff, xlen, 0))
+                long_evict<true>(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e, ls);
+            continue;
+        }
+        if (xfront) {
+            const int xsd = __shfl_sync(0xffffffffu, sd, src);
+            const bool spec = expand_early(P);
+            if (!hub || !make_hub(C, P, xv, spec ? HUB_FRONT_SPEC : HUB_FRONT, xk, xoff, xlen, spec ? xsd : 0))
+                long_front(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e, ls);
+            continue;
+        }
+        unsigned long long q = 0;
+        if (rec_of(__shfl_sync(0xffffffffu, rec, src), e, q)) {
+            const int cnt = __ldcg(P.arena + 4 * q);
+            if (P.hub_len > 0 && cnt >= P.hub_len &&
+                make_hub(C, P, xv, HUB_EVICT_REC, xk, (long long)(4 * q + 4), cnt, 0))
+                continue;
+            act_recorded(g, C, P, B, W, P.arena + 4 * q + 4, 0, cnt, xk);
+            if (lane == 0) {
+                ls.ev++;
+                ls.evl += cnt;
+            }
+        } else if (!hub || !make_hub(C, P, xv, HUB_EVICT_INS, xk, xoff, xlen, 0)) {
+            long_evict<false>(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e, ls);
+        }
+    }
+    publish_records(P, W, e);
+    // the others together, up to 128 quads a window
+    unsigned rest = __ballot_sync(0xffffffffu, vert && len <= kShort);
+    if (!rest) return;
+    if ((rest & (rest - 1)) == 0) {   // one: searches spend their thin phases here, so take the fewest steps
+        const int src = __ffs(rest) - 1;
+        lone_short<DEL>(g, C, P, B, W, __shfl_sync(0xffffffffu, v, src), __shfl_sync(0xffffffffu, k, src),
+                        g.adj + __shfl_sync(0xffffffffu, off, src), __shfl_sync(0xffffffffu, len, src),
+                        __shfl_sync(0xffffffffu, (int)front, src) != 0, e, ls);
+        return;
+    }
+    const int nq = vert && len <= kShort ? (len + 3) >> 2 : 0;
+    int incl = nq;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    int gbase = 0;
+    while (rest) {
+        const bool in = ((rest >> lane) & 1u) && incl - gbase <= 128;   // at least one: a list has <= 32 quads
+        const unsigned gm = __ballot_sync(0xffffffffu, in);
+        const int gend = __shfl_sync(0xffffffffu, incl, 31 - __clz(gm));
+        B.csd[lane] = 0;
+        __syncwarp();
+        int id[16];
+        uint32_t key[16];
+        unsigned owners = 0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int q = gbase + u * 32 + lane;
+            int o = 0;   // the owner: the first lane whose running quad count exceeds q
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(0xffffffffu, incl, o + step - 1) <= q) o += step;
+            const long long ob = __shfl_sync(0xffffffffu, off, o);
+            const int ol = __shfl_sync(0xffffffffu, len, o);
+            const int t0 = (q - __shfl_sync(0xffffffffu, incl - nq, o)) * 4;
+            owners |= (unsigned)o << (8 * u);
+            int4 a = make_int4(HOLE, HOLE, HOLE, HOLE);
+            if (q < gend) a = __ldcs(reinterpret_cast<const int4*>(g.adj + ob + t0));
+            id[4 * u] = a.x;
+            id[4 * u + 1] = t0 + 1 < ol ? a.y : HOLE;
+            id[4 * u + 2] = t0 + 2 < ol ? a.z : HOLE;
+            id[4 * u + 3] = t0 + 3 < ol ? a.w : HOLE;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; i++) key[i] = id[i] >= 0 ? g.kc[id[i]] : KEY_DEAD;
+        unsigned mask = 0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int o = (int)((owners >> (8 * u)) & 31u);
+            const int kk = __shfl_sync(0xffffffffu, k, o);
+            int part = 0;
+#pragma unroll
+            for (int i = 4 * u; i < 4 * u + 4; i++) {
+                if (DEL) {
+                    mask |= key_core(key[i]) == kk ? 1u << i : 0u;
+                } else {
+                    part += (int)key[i] >= 2 * kk + 1;
+                    mask |= key[i] == (uint32_t)(2 * kk + 1) ? 1u << i : 0u;
+                }
+            }
+            if (!DEL && part) atomicAdd(&B.csd[o], part);
+        }
+        const int cnt = __popc(mask);
+        int cinc = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, cinc, o);
+            if (lane >= o) cinc += x;
+        }
+        const int nc = __shfl_sync(0xffffffffu, cinc, 31);
+        int at = cinc - cnt;
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            if ((mask >> i) & 1u) {
+                B.id[at] = id[i];
+                B.own[at++] = (uint8_t)((owners >> (8 * (i >> 2))) & 31u);
+            }
+        }
+        __syncwarp();
+        if (DEL) {
+            act_delete<true>(g, C, P, B, W, nc, k, e);
+            if (in) {
+                g.hc[v].x = k - 1;
+                g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
+                ls.ev++;
+                ls.evl += len;
+            }
+        } else {
+            int csd = 0;
+            unsigned long long old = 0;
+            if (in && front) {
+                csd = B.csd[lane];
+                old = add_csd(g, v, csd);
+                ls.vis++;
+                ls.visl += len;
+            } else if (in) {
+                ls.ev++;
+                ls.evl += len;
+            }
+            act_insert<true>(g, C, P, B, W, nc, k, e, [&] {
+                const bool up = in && front && ww(old) + csd > k;
+                if (in && front && !up) ls.ev++;
+                return __ballot_sync(0xffffffffu, up);
+            });
+        }
+        __syncwarp();
+        rest &= ~gm;
+        gbase = gend;
+    }
+}
+
+// Search (iteration number) whose queue the block's poller found quiescent.
+__shared__ volatile uint32_t s_quiet;
+
+// Drains the task queue (every warp of the grid).  Returns false on error.
+// A warp claims slots for its lanes with one atomic and polls them together;
+// it runs whatever is ready as one batch.  How many it claims follows the
+// queue's backlog when it last claimed: one slot when tasks are scarce (a
+// slot past the tail is waited for), its share when they are plenty, at most
+// 32 (P.claim_max raises the share it takes; guided self-scheduling, so that
+// the last tasks of a search still spread over all warps).  Finished tasks
+// are reported in batches, always before the warp waits on an empty slot (so
+// a waiting warp never holds back the quiescence test).  Inlined into the
+// kernel: as a separate function it took the graph and the parameters by
+// reference, which put both in local memory.
+template <bool DEL>
+__device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const MaintainParams& P, uint32_t e,
+                                             LocalStats& ls) {
+    const int lane = lane_id();
+    WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
+    const unsigned long long t_start = gtimer();
+    const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+    const unsigned long long share = (unsigned long long)(P.claim_max > 1 ? P.claim_max : 1);
+    unsigned long long idx = 0, ndone = 0;
+    unsigned held = 0;   // lanes that hold a claimed slot
+    int claim = 1;
+    unsigned int nap = 32;
+    Walker W{0, 1, 0, 0, 0ull, 0ull, 0ull};
+    // one warp per block tests quiescence and tells the others through
+    // shared memory: a test reads two hot counters, and thousands of
+    // waiting warps reading them would slow the claims and pushes that
+    // share those counters' L2 slices
+    const bool poller = threadIdx.x < 32;
+    for (unsigned int spins = 0;; spins++) {
+        unsigned long long t = TASK_EMPTY, h = 0, tl = 0;
+        bool look = false;   // the backlog was read in this round
+        if (W.nk > 0) {      // the tasks this warp kept
+            if (lane < W.nk) t = B.kept[lane];
+            __syncwarp();
+            W.nk = 0;
+            if (W.klim > 1) {
+                look = true;
+                h = lane == 0 ? vload64(&C->task_head) : 0ull;
+                tl = lane == 1 ? vload64(&C->task_tail) : 0ull;
+            }
+        } else {
+            if (!held) {
+                if (lane == 0) h = atomicAdd(&C->task_head, (unsigned long long)claim);
+                else if (lane == 1) tl = vload64(&C->task_tail);
+                look = true;
+                held = claim == 32 ? 0xffffffffu : (1u << claim) - 1u;
+                idx = __shfl_sync(0xffffffffu, h, 0) + (unsigned long long)lane;
+            }
+            unsigned long long* slot = &P.TQ[idx & P.tqmask];
+            const bool mine = (held >> lane) & 1u;
+            if (mine) t = vload64(slot);
+            const unsigned got = __ballot_sync(0xffffffffu, t != TASK_EMPTY);
+            if (!got) {
+                int quit = 0;
+                if (lane == 0) {
+                    if (ndone) {   // report before waiting
+                        __threadfence();
+                        atomicAdd(&C->task_done, ndone);
+                    }
+                    if (poller) {
+                        // quiescent: every task pushed has finished (done read first)
+                        const unsigned long long d = ld_acquire64(&C->task_done);   // read before the tail
+                        if (d == vload64(&C->task_tail) || vload32(&C->error)) {
+                            s_quiet = e;
+                            quit = 1;
+                        }
+                    } else if (s_quiet == e) {
+                        quit = 1;
+                    }
+                    if (!quit && (spins & 3u) == 0 && gtimer() - t_start > P.limit_ns) {
+                        atomicCAS(&C->error, 0, E_BARRIER_TIMEOUT);
+                        quit = 1;
+                    }
+                }
+                ndone = 0;
+                if (__shfl_sync(0xffffffffu, quit, 0)) break;
+                __nanosleep(nap);
+                if (nap < 512) nap <<= 1;
+                claim = 1;
+                W.klim = 1;
+                continue;
+            }
+            nap = 32;
+            if (t != TASK_EMPTY) vstore64(slot, TASK_EMPTY);   // free for the next search
+            held &= ~got;
+            ndone += (unsigned long long)__popc(got);
+        }
+        // acquire: a deletion's tasks need the cores and change stamps as their
+        // producers left them (measured necessary: without it, warps running
+        // several claimed tasks in a row reached wrong cores on small delete
+        // batches), a chunk task its hub item.  An insertion's search changes
+        // nothing of a vertex but its per-iteration word, which is only ever
+        // read and updated at L2, and its record, which is read with acquire.
+        if (DEL || __any_sync(0xffffffffu, t != TASK_EMPTY && (int)(t >> 62) == T_CHUNK)) __threadfence();
+        run_batch<DEL>(g, C, P, B, W, e, ls, t);
+        __syncwarp();
+        if (look) {
+            h = __shfl_sync(0xffffffffu, h, 0);
+            tl = __shfl_sync(0xffffffffu, tl, 1);
+            const unsigned long long backlog = tl > h ? tl - h : 0ull;
+            const unsigned long long c = backlog * share / (2 * nwarps);
+            claim = c < 1 ? 1 : c > 32 ? 32 : (int)c;
+            W.klim = backlog > 2 * nwarps ? 32 : 1;
+        }
+    }
+    return vload32(&C->error) == 0;
+}
+
+// Queues tasks for log entries [lo, hi) that are already in the log (a
+// search resumed from the single-block mode).  Every warp calls it.
+__device__ __forceinline__ void seed_tasks(Ctl* C, const MaintainParams& P, const int32_t* log, unsigned long long lo,
+                                           unsigned long long hi, int type) {
+    const int lane = lane_id();
+    const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (unsigned long long base = lo + (unsigned long long)gwarp * 32; base < hi;
+         base += (unsigned long long)nwarps * 32) {
+        const unsigned long long cnt = min(32ull, hi - base);
+        unsigned long long tb = 0;
+        if (lane == 0) tb = atomicAdd(&C->task_tail, cnt);
+        tb = __shfl_sync(0xffffffffu, tb, 0);
+        if (task_room(C, P, tb, cnt) && (unsigned long long)lane < cnt)
+            vstore64(&P.TQ[(tb + lane) & P.tqmask],
+                     mk_task(type, (unsigned long long)(uint32_t)log[(base + lane) & P.qmask]));
+    }
+}
+
+}  // namespace cm

@@ -198,7 +198,7 @@ struct BlockGroup {
 constexpr unsigned long long TASK_EMPTY = ~0ull;
 enum { T_FRONT = 0, T_EVICT = 1, T_CHUNK = 2 };
 constexpr int kTaskChunkBits = 22;          // chunk index within a hub item
-constexpr unsigned long long kTaskMargin = 1ull << 16;   // slots kept free for claims past the tail
+constexpr unsigned long long kTaskMargin = 1ull << 18;   // slots kept free for claims past the tail (32 per warp)
 
 __device__ __forceinline__ unsigned long long mk_task(int type, unsigned long long payload) {
     return ((unsigned long long)type << 62) | payload;
@@ -213,35 +213,19 @@ __device__ __forceinline__ bool task_room(Ctl* C, const MaintainParams& P, unsig
     return true;
 }
 
-// The task a warp keeps for itself (grid mode).  Of the vertices a warp
-// produces in the last scan step of its current task, the first is not
-// queued: the warp runs it next, which saves the hand-off through the queue
-// (the slot write, another warp's poll and its back-off) on every level of a
-// dependency chain, such as a frontier vertex that fails and evicts itself or
-// an eviction that evicts a neighbour.  The kept task is not counted in the
-// queue's tail and is not reported done; the task that produced it is
-// reported only after the warp has run it, so quiescence still waits for it.
-constexpr int kGridWarps = 16;   // warps per grid-mode block
-__shared__ unsigned long long s_keep[kGridWarps];
-__device__ __forceinline__ unsigned long long& kept_task() { return s_keep[threadIdx.x >> 5]; }
-
-// Pushes the vertices of the lanes with pred set (warp-collective).  keep:
-// this is the task's last scan step, so the warp may keep one of them.
+// Pushes the vertices of the lanes with pred set (warp-collective).
 template <bool ASYNC>
-__device__ __forceinline__ void push_vertex(Ctl* C, const MaintainParams& P, bool pred, int32_t v, int which,
-                                            bool keep = false) {
+__device__ __forceinline__ void push_vertex(Ctl* C, const MaintainParams& P, bool pred, int32_t v, int which) {
     // which 0: frontier (VQ, T_FRONT), 1: eviction (EQ, T_EVICT)
     const unsigned int b = __ballot_sync(0xffffffffu, pred);
     if (!b) return;
     const int lane = lane_id();
     const int leader = __ffs(b) - 1;
     const unsigned long long cnt = (unsigned long long)__popc(b);
-    if (ASYNC) keep = keep && kept_task() == TASK_EMPTY;   // the same value in every lane
-    const unsigned long long nq = cnt - (ASYNC && keep ? 1 : 0);
     unsigned long long lb = 0, tb = 0;
     if (lane == leader) {
         lb = atomicAdd(&C->tail[which], cnt);
-        if (ASYNC && nq) tb = atomicAdd(&C->task_tail, nq);
+        if (ASYNC) tb = atomicAdd(&C->task_tail, cnt);
     }
     lb = __shfl_sync(0xffffffffu, lb, leader);
     const unsigned int rank = __popc(b & ((1u << lane) - 1));
@@ -250,18 +234,14 @@ __device__ __forceinline__ void push_vertex(Ctl* C, const MaintainParams& P, boo
     if (ASYNC) {
         tb = __shfl_sync(0xffffffffu, tb, leader);
         const unsigned long long task = mk_task(which == 0 ? T_FRONT : T_EVICT, (unsigned long long)v);
-        const bool room = nq == 0 || task_room(C, P, tb, nq);
-        if (pred && keep && rank == 0) kept_task() = task;
-        else if (pred && room) vstore64(&P.TQ[(tb + rank - (keep ? 1 : 0)) & P.tqmask], task);
-        __syncwarp();
+        if (task_room(C, P, tb, cnt) && pred) vstore64(&P.TQ[(tb + rank) & P.tqmask], task);
     }
 }
 
-// The same for up to four vertices per lane (one scan step), with one
-// atomic per queue for the whole warp.
-template <bool ASYNC>
+// Appends up to four vertices per lane (one scan step of a wave) to a log,
+// with one atomic for the whole warp.
 __device__ __forceinline__ void push_vertex4(Ctl* C, const MaintainParams& P, const bool pred[4], const int32_t v[4],
-                                             int which, bool keep = false) {
+                                             int which) {
     const int lane = lane_id();
     const int mine = (int)pred[0] + (int)pred[1] + (int)pred[2] + (int)pred[3];
     if (!__any_sync(0xffffffffu, mine != 0)) return;
@@ -272,33 +252,14 @@ __device__ __forceinline__ void push_vertex4(Ctl* C, const MaintainParams& P, co
         if (lane >= o) incl += t;
     }
     const unsigned long long total = (unsigned long long)__shfl_sync(0xffffffffu, incl, 31);
-    if (ASYNC) keep = keep && kept_task() == TASK_EMPTY;
-    const unsigned long long nq = total - (ASYNC && keep ? 1 : 0);
-    unsigned long long lb = 0, tb = 0;
-    if (lane == 31) {
-        lb = atomicAdd(&C->tail[which], total);
-        if (ASYNC && nq) tb = atomicAdd(&C->task_tail, nq);
-    }
+    unsigned long long lb = 0;
+    if (lane == 31) lb = atomicAdd(&C->tail[which], total);
     lb = __shfl_sync(0xffffffffu, lb, 31);
     unsigned long long at = (unsigned long long)(incl - mine);
     int32_t* log = which == 0 ? P.VQ : P.EQ;
-    bool room = true;
-    if (ASYNC) {
-        tb = __shfl_sync(0xffffffffu, tb, 31);
-        room = nq == 0 || task_room(C, P, tb, nq);
-    }
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        if (!pred[q]) continue;
-        log[(lb + at) & P.qmask] = v[q];
-        if (ASYNC) {
-            const unsigned long long task = mk_task(which == 0 ? T_FRONT : T_EVICT, (unsigned long long)v[q]);
-            if (keep && at == 0) kept_task() = task;
-            else if (room) vstore64(&P.TQ[(tb + at - (keep ? 1 : 0)) & P.tqmask], task);
-        }
-        at++;
-    }
-    if (ASYNC) __syncwarp();
+    for (int q = 0; q < 4; q++)
+        if (pred[q]) log[(lb + at++) & P.qmask] = v[q];
 }
 
 // The words of a scan step's four neighbours as {core, SD, z, w}.  First
@@ -348,8 +309,7 @@ __device__ __forceinline__ void load4(const DevGraph& g, long long o, int len, i
 // 16-byte words of two consecutive steps before the first step's gathers,
 // so a step's neighbour gathers do not wait behind its own list read.  List
 // reads are streamed (evict-first) so that L2 keeps the per-vertex keys.
-// Inside, `int w[4]` holds the step's four neighbour ids (HOLE past s1)
-// and `last_` is set in the group's last step.
+// Inside, `int w[4]` holds the step's four neighbour ids (HOLE past s1).
 #define SCANP_RANGE(Grp, o, s0, s1)                                                              \
     for (int blk_ = (s0) + Grp::first() * 4; blk_ < (s1); blk_ += Grp::G * 8) {                  \
         int4 A_[2];                                                                               \
@@ -361,7 +321,6 @@ __device__ __forceinline__ void load4(const DevGraph& g, long long o, int len, i
         _Pragma("unroll") for (int j_ = 0; j_ < 2; j_++) {                                         \
             if (blk_ + j_ * Grp::G * 4 >= (s1)) break;                                            \
             const int t0_ = blk_ + j_ * Grp::G * 4 + lane_id() * 4;                               \
-            const bool last_ = blk_ + (j_ + 1) * Grp::G * 4 >= (s1);                              \
             int w[4];                                                                             \
             w[0] = A_[j_].x;                                                                      \
             w[1] = t0_ + 1 < (s1) ? A_[j_].y : HOLE;                                              \
@@ -372,9 +331,9 @@ __device__ __forceinline__ void load4(const DevGraph& g, long long o, int len, i
     }
 
 // ---------------------------------------------------------------- range scans
-// Each scan covers slots [s0, s1) of the list at offset o of a vertex at
-// level k, so a vertex can be scanned whole by one group or in chunks by
-// many blocks.
+// Scans of the wave mode (one block) and of the SD fix-up: slots [s0, s1) of
+// the list at offset o of a vertex at level k.  (The grid mode's search has
+// its own scans, in cm_search.cuh.)
 
 // This thread's part of CSD over the range (Definition 8 with the SD of
 // Definition 7: neighbours above k, and core-k neighbours with SD > k).
@@ -393,7 +352,7 @@ __device__ __forceinline__ int csd_part(const DevGraph& g, int k, long long o, i
 
 // Visits the unvisited core-k neighbours with SD > k in the range and
 // appends them to the next frontier.
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ void expand_range(const DevGraph& g, Ctl* C, const MaintainParams& P, int k, long long o,
                                              int s0, int s1, uint32_t e) {
     SCANP_RANGE(Grp, o, s0, s1)
@@ -408,7 +367,7 @@ __device__ __forceinline__ void expand_range(const DevGraph& g, Ctl* C, const Ma
             sw[q] = word_of(h[q]);
         }
         visit4(g, C, w, p, e, sw);
-        push_vertex4<ASYNC>(C, P, p, w, 0, last_);
+        push_vertex4(C, P, p, w, 0);
     SCANP_END
 }
 
@@ -416,7 +375,7 @@ __device__ __forceinline__ void expand_range(const DevGraph& g, Ctl* C, const Ma
 // range's unvisited core-k neighbours with SD > k in the same pass: the
 // expansion of Algorithm 3 done before the vertex's support is known
 // (speculative expansion, see process_frontier).
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ int csd_expand_range(const DevGraph& g, Ctl* C, const MaintainParams& P, int k,
                                                 long long o, int s0, int s1, uint32_t e) {
     int pcd = 0;
@@ -433,7 +392,7 @@ __device__ __forceinline__ int csd_expand_range(const DevGraph& g, Ctl* C, const
             sw[q] = word_of(h[q]);
         }
         visit4(g, C, w, p, e, sw);
-        push_vertex4<ASYNC>(C, P, p, w, 0, last_);
+        push_vertex4(C, P, p, w, 0);
     SCANP_END
     return pcd;
 }
@@ -447,16 +406,12 @@ __device__ __forceinline__ int csd_expand_range(const DevGraph& g, Ctl* C, const
 // cores are the same (see the design notes).  On R-MAT sweeps the visited
 // vertices grow by about 1.5% and the inserts get up to 20% faster, so it
 // is the default; expand_early = -1 restores the paper's order.
-__device__ __forceinline__ bool expand_early(const MaintainParams& P, int sd, int k) {
-    (void)sd;
-    (void)k;
-    return P.expand_early >= 0;
-}
+__device__ __forceinline__ bool expand_early(const MaintainParams& P) { return P.expand_early >= 0; }
 
 // InsertRemove over the range (Algorithm 4): every core-k neighbour with
 // SD > k (visited or not) loses one support; a processed one whose support
 // falls to k leaves too.
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ void evict_ins_range(const DevGraph& g, Ctl* C, const MaintainParams& P, int k,
                                                 long long o, int s0, int s1, uint32_t e) {
     SCANP_RANGE(Grp, o, s0, s1)
@@ -475,14 +430,14 @@ __device__ __forceinline__ void evict_ins_range(const DevGraph& g, Ctl* C, const
         add_word4(g, C, w, cand, e, -1, sw, of, oc);
 #pragma unroll
         for (int q = 0; q < 4; q++) p[q] = cand[q] && (of[q] & kProcessed) && oc[q] == k + 1;
-        push_vertex4<ASYNC>(C, P, p, w, 1, last_);
+        push_vertex4(C, P, p, w, 1);
     SCANP_END
 }
 
 // DeleteRemove over the range (Algorithm 7): each core-k neighbour w loses
 // one support (initially SD(w)) and leaves when it falls below k, i.e. when
 // its count of evicted neighbours reaches SD(w) - k + 1.
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ void evict_del_range(const DevGraph& g, Ctl* C, const MaintainParams& P, int k,
                                                 long long o, int s0, int s1, uint32_t e) {
     SCANP_RANGE(Grp, o, s0, s1)
@@ -510,7 +465,7 @@ __device__ __forceinline__ void evict_del_range(const DevGraph& g, Ctl* C, const
             p[q] = cand[q] && oc[q] + 1 == h[q].y - k + 1;
             if (p[q]) g.chg[w[q]] = e;
         }
-        push_vertex4<ASYNC>(C, P, p, w, 1, last_);
+        push_vertex4(C, P, p, w, 1);
     SCANP_END
 }
 
@@ -535,7 +490,7 @@ __device__ __forceinline__ VInfo load_vinfo(const DevGraph& g, int v) {
 // Positive search step (Algorithm 3) for a frontier vertex v at level k:
 // support += CSD(v); above k -> visit the unvisited core-k neighbours with
 // SD > k, else v is evicted.
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ void process_frontier(const DevGraph& g, Ctl* C, const MaintainParams& P, int v,
                                                  const VInfo& vi, uint32_t e, LocalStats& ls) {
     const int lane = lane_id();
@@ -572,15 +527,15 @@ __device__ __forceinline__ void process_frontier(const DevGraph& g, Ctl* C, cons
                     sw[q] = word_of(h[q]);
                 }
                 visit4(g, C, w, p, e, sw);
-                push_vertex4<ASYNC>(C, P, p, w, 0, true);
+                push_vertex4(C, P, p, w, 0);
             } else {
-                push_vertex<ASYNC>(C, P, lane == 0, v, 1, true);
+                push_vertex<false>(C, P, lane == 0, v, 1);
             }
             return;
         }
     }
-    const bool early = expand_early(P, vi.h.y, k);
-    const int pcd = Grp::sum(early ? csd_expand_range<Grp, ASYNC>(g, C, P, k, o, 0, len, e)
+    const bool early = expand_early(P);
+    const int pcd = Grp::sum(early ? csd_expand_range<Grp>(g, C, P, k, o, 0, len, e)
                                    : csd_part<Grp>(g, k, o, 0, len));
     int32_t sup = 0;
     if (Grp::rank0()) {
@@ -597,18 +552,18 @@ __device__ __forceinline__ void process_frontier(const DevGraph& g, Ctl* C, cons
         sup = Grp::sum(Grp::rank0() ? sup : 0);
     }
     if (sup > k) {
-        if (!early) expand_range<Grp, ASYNC>(g, C, P, k, o, 0, len, e);
+        if (!early) expand_range<Grp>(g, C, P, k, o, 0, len, e);
     } else if (Grp::warp0()) {
-        push_vertex<ASYNC>(C, P, lane == 0, v, 1, Grp::G == 32);
+        push_vertex<false>(C, P, lane == 0, v, 1);
     }
 }
 
 // InsertRemove step (Algorithm 4) for an evicted vertex v.
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ void evict_insert_vertex(const DevGraph& g, Ctl* C, const MaintainParams& P,
                                                     const VInfo& vi, uint32_t e, LocalStats& ls) {
     const int len = vi.len;
-    evict_ins_range<Grp, ASYNC>(g, C, P, vi.h.x, vi.o, 0, len, e);
+    evict_ins_range<Grp>(g, C, P, vi.h.x, vi.o, 0, len, e);
     if (Grp::rank0()) {
         ls.ev++;
         ls.evl += len;
@@ -616,12 +571,12 @@ __device__ __forceinline__ void evict_insert_vertex(const DevGraph& g, Ctl* C, c
 }
 
 // DeleteRemove step (Algorithm 7) for an evicted vertex v, which drops to k-1.
-template <class Grp, bool ASYNC>
+template <class Grp>
 __device__ __forceinline__ void evict_delete_vertex(const DevGraph& g, Ctl* C, const MaintainParams& P, int v,
                                                     const VInfo& vi, uint32_t e, LocalStats& ls) {
     const int k = vi.h.x;
     const int len = vi.len;
-    evict_del_range<Grp, ASYNC>(g, C, P, k, vi.o, 0, len, e);
+    evict_del_range<Grp>(g, C, P, k, vi.o, 0, len, e);
     if constexpr (Grp::G > 32) __syncthreads();   // every warp has read k before it changes
     if (Grp::rank0()) {
         g.hc[v].x = k - 1;
