@@ -364,17 +364,17 @@ static int ensure_batch(cm_graph* h, long long k) {
 }
 
 // ------------------------------------------------------------------ launch geometry
-// Persistent kernels fill max_sms SMs (all by default) with as many blocks
-// as stay resident.  A small batch gets fewer blocks: grid barriers then
+// The maintenance kernel fills max_sms SMs (all by default) with as many
+// blocks as stay resident.  A small batch gets fewer blocks: grid barriers then
 // cost less, and there is not enough work for the whole GPU anyway.
-static void persistent_geometry(cm_graph* h, int kind, long long work, int* blocks, int* threads) {
-    const int t = 512;   // both persistent kernels run 512-thread blocks
-    int occ = kind == 0 ? maintain_blocks_per_sm(t) : peel_blocks_per_sm(t);
+static void persistent_geometry(cm_graph* h, long long work, int* blocks, int* threads) {
+    const int t = kGridThreadsHost;
+    int occ = maintain_blocks_per_sm(t);
     if (occ < 1) occ = 1;
     int bps = h->opt.blocks_per_sm > 0 ? (h->opt.blocks_per_sm < occ ? h->opt.blocks_per_sm : occ) : occ;
     int sms = h->opt.max_sms > 0 && h->opt.max_sms < h->num_sms ? h->opt.max_sms : h->num_sms;
     long long b = (long long)sms * bps;
-    if (kind == 0 && h->opt.blocks_per_sm <= 0) {
+    if (h->opt.blocks_per_sm <= 0) {
         long long want = (work * 64 + t - 1) / t;
         if (want < sms) want = sms;
         if (want < b) b = want;
@@ -610,28 +610,29 @@ static int peel_all(cm_graph* h) {
     p.g.n = h->n;
     p.ctl = h->ctl;
     p.dcur = h->CQ;
-    p.L0 = h->VQ;
-    p.L1 = h->EQ;
-    p.F = h->OVL;
-    p.qmask = h->qmask;
+    p.list = h->VQ;   // the rings are powers of two >= the vertex capacity (>= 1,024)
+    p.far = h->OVL;
     // the hub-item ring is scratch outside a maintenance search
     p.chunks = reinterpret_cast<unsigned long long*>(h->HQ);
     p.chunk_cap = kHubRing * sizeof(HubItem) / sizeof(unsigned long long);
     p.limit_ns = (unsigned long long)h->opt.spin_limit_ns;
-    int blocks, threads;
-    persistent_geometry(h, 1, h->n, &blocks, &threads);
-    p.expect = (uint32_t)blocks;
-    LAUNCH(h, launch_peel(p, blocks, threads, h->stream));
+    // one block per SM (of max_sms); fewer for a small graph, whose barriers
+    // then cost less (a block scans at least 256 vertices)
+    long long blocks = h->opt.max_sms > 0 && h->opt.max_sms < h->num_sms ? h->opt.max_sms : h->num_sms;
+    if (blocks > 1000) blocks = 1000;   // the barrier word counts to 1,023
+    if (blocks > ((long long)h->n + 255) / 256) blocks = ((long long)h->n + 255) / 256;
+    if (blocks < 1) blocks = 1;
+    LAUNCH(h, launch_peel(p, (int)blocks, h->stream));
     if ((rc = rd_ctl(h))) return rc;
     if (h->hctl->error) {
         h->poisoned = true;
         return set_err(h, CM_ERR_LIMIT, "peeling stopped with device error %d", h->hctl->error);
     }
     h->last.peel_levels = (int64_t)h->hctl->st[ST_LEVELS];
-    h->last.waves = (int64_t)h->hctl->st[ST_WAVES];   // sub-waves of the peel
+    h->last.waves = (int64_t)h->hctl->st[ST_WAVES];   // levels, and sub-waves of work the grid shared
     h->last.barriers = (int64_t)h->hctl->st[ST_BARRIERS];
-    // phase times of the peel: level scans, sub-waves, chunk phases
-    for (int i = 0; i < 3; i++) h->last.phase_ns[i] = (int64_t)h->hctl->ph[i];
+    // phase times of the peel: levels (scan and cascades), shared sub-waves
+    for (int i = 0; i < 2; i++) h->last.phase_ns[i] = (int64_t)h->hctl->ph[i];
     // Algorithmic bytes of the peel: 16 B per vertex to start it (degree
     // read, working degree, core and list writes); 12 B per remaining-list
     // entry scanned at a level (id, working degree, list write); 12 B per
@@ -835,7 +836,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         MaintainParams p = handle_params(h, op);
         p.max_iters = nrem0 + 1;
         int blocks, threads;
-        persistent_geometry(h, 0, nrem0, &blocks, &threads);
+        persistent_geometry(h, nrem0, &blocks, &threads);
         p.expect = (uint32_t)blocks;
         bool debug_hang = (h->opt.debug_flags & CM_DEBUG_BARRIER_NEVER_RELEASES) != 0;
         if (debug_hang) {

@@ -132,8 +132,10 @@ struct __align__(128) Ctl {
     unsigned long long spc[kTails];    // snapshot of pc at the last barrier
     unsigned long long st[ST_COUNT];
     unsigned long long ph[PH_COUNT];   // nanoseconds per phase (block 0's view)
+    alignas(128) unsigned long long pw[4];          // peel: barrier words (cm_peel.cuh)
+    unsigned long long pm[4];                       // peel: 0x7FFFFFFF - smallest degree kept at a level
     // ingest / host exchange
-    unsigned long long nrem;       // edges kept by ingest
+    alignas(128) unsigned long long nrem;       // edges kept by ingest
     unsigned long long noverflow;  // vertices whose capacity the batch exceeds
     unsigned long long reloc_need; // slots needed to relocate them
     unsigned long long adj_top;    // bump pointer of the adjacency pool

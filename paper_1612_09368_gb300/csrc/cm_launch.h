@@ -57,14 +57,10 @@ struct PeelParams {
     DevGraph g;
     Ctl* ctl;
     int32_t* dcur;    // working degree [n]
-    int32_t* L0;      // remaining-vertex lists [n]
-    int32_t* L1;
-    int32_t* F;       // frontier ring [qmask+1]
-    unsigned long long qmask;
-    unsigned long long* chunks;     // chunk tasks of high-degree frontier vertices
+    int32_t* list;    // remaining vertices [n rounded up to 32]
+    int32_t* far;     // vertices handed to the grid [n]
+    unsigned long long* chunks;     // chunk tasks of long lists
     unsigned long long chunk_cap;
-    uint32_t expect;
-    uint32_t pad;
     unsigned long long limit_ns;
 };
 
@@ -102,8 +98,7 @@ cudaError_t scatter_edges(const int32_t* E, const uint32_t* ebkt, long long m, D
 cudaError_t set_cores(const int32_t* cores, DevGraph g, cudaStream_t s);
 // core_scratch: n int32 of scratch (receives a compact copy of the cores)
 cudaError_t init_mcd(DevGraph g, int32_t v0, int32_t v1, int32_t* core_scratch, cudaStream_t s);
-cudaError_t launch_peel(const PeelParams& p, int blocks, int threads, cudaStream_t s);
-int peel_blocks_per_sm(int threads);
+cudaError_t launch_peel(const PeelParams& p, int blocks, cudaStream_t s);
 cudaError_t rehash(const Bucket* old_idx, unsigned long long old_size, DevGraph g, Ctl* c, cudaStream_t s);
 cudaError_t validate_vertices(const int64_t* nbr_off, const int32_t* nbrs, int32_t count, int32_t base, DevGraph g,
                               Ctl* c, cudaStream_t s);

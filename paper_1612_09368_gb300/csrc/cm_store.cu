@@ -3,11 +3,11 @@
 // export.
 #include "cm_common.cuh"
 #include "cm_launch.h"
+#include "cm_peel.cuh"
 
 namespace cm {
 
 constexpr uint32_t BKT_DROP = 0xFFFFFFFFu;
-constexpr int UNPEELED = -2;
 
 static inline unsigned grid_for(long long n, int t, long long cap = 1 << 20) {
     long long b = (n + t - 1) / t;
@@ -170,373 +170,38 @@ cudaError_t init_mcd(DevGraph g, int32_t v0, int32_t v1, int32_t* core_scratch, 
 }
 
 // ------------------------------------------------------------------ peeling
-// Level-synchronous bucket peeling (the static O(m) decomposition the paper
-// cites, run level by level): at level k every remaining vertex whose
-// degree is <= k gets core k and leaves; each departure takes one degree
-// from every remaining neighbour, and neighbours that reach k leave at the
-// same level.  Empty levels are skipped to the smallest remaining degree.
-//
-// Working degrees only fall, one at a time, and a vertex leaves at level k
-// exactly when its degree reaches k (the decrement from k + 1 to k, or the
-// level's scan finding it at k).  So at the scan of level k every remaining
-// vertex has degree >= k and every vertex that left has degree < k: the
-// scan reads the working degree alone (never the vertex's {core, SD} word)
-// to tell the three cases apart.
-//
-// A frontier vertex with at least kPeelBig slots is not scanned by the warp
-// that takes it: its list is cut into kPeelChunk-slot chunk tasks that every
-// warp takes after a barrier, so one high-degree vertex does not hold a whole
-// sub-wave on a single warp.
-//
-// No counter is shared by the whole grid per vertex: the level scan
-// compacts a tile of kScanTile entries per block in shared memory and
-// appends it with one atomic per list; frontier vertices and chunk tasks
-// are dealt to warps by index, not claimed; and the vertices a sub-wave
-// peels collect in a per-warp shared buffer that reaches the frontier ring
-// with one atomic per flush.  (With one atomic per warp per step on a few
-// counters, the serialised atomics at those counters were most of the
-// peel's time.)
-constexpr int kPeelThreads = 512;
-constexpr int kPeelWarps = kPeelThreads / 32;
-constexpr int kPeelBig = 2048;
-constexpr int kPeelChunk = 512;
-constexpr unsigned long long kPeelNoTask = ~0ull;
-constexpr int kScanTile = 4 * kPeelThreads;   // list entries per block and scan step
-constexpr int kPushBuf = 256;                 // per-warp buffer of peeled vertices
-constexpr int kPushFlush = kPushBuf - 128;    // a scan step adds at most 128
-
-struct PeelShared {
-    int32_t keep[kScanTile];            // level scan: survivors of the tile
-    int32_t peel[kScanTile];            // level scan: vertices of degree k
-    int32_t buf[kPeelWarps][kPushBuf];  // sub-waves: peeled vertices per warp
-    int wcnt[kPeelWarps];
-    int nkeep, npeel, mx;
-    unsigned long long kbase, pbase, wbase;
-};
-
-// Appends the warp's buffered vertices to the frontier ring (one atomic).
-__device__ __forceinline__ void flush_peeled(Ctl* C, const PeelParams& P, int32_t* buf, int& cnt) {
-    if (cnt == 0) return;
-    unsigned long long b = 0;
-    if (lane_id() == 0) b = atomicAdd(&C->tail[0], (unsigned long long)cnt);
-    b = __shfl_sync(0xffffffffu, b, 0);
-    for (int i = lane_id(); i < cnt; i += 32) P.F[b + i] = buf[i];
-    __syncwarp();
-    cnt = 0;
-}
-
-// End of a sub-wave: the block's warps append their buffers to the frontier
-// ring together, with one atomic.  Every thread of the block calls it.
-__device__ __forceinline__ void block_flush_peeled(Ctl* C, const PeelParams& P, PeelShared& S, int& cnt) {
-    const int wib = threadIdx.x >> 5;
-    if (lane_id() == 0) S.wcnt[wib] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int tot = 0;
-        for (int i = 0; i < kPeelWarps; i++) tot += S.wcnt[i];
-        S.wbase = tot ? atomicAdd(&C->tail[0], (unsigned long long)tot) : 0;
+// The store as cm_peel.cuh reads it: lists start 16-byte aligned, their
+// capacity is a multiple of 4 (so a quad never leaves the list's
+// allocation) and deleted entries are holes.
+struct PeelStore {
+    DevGraph d;
+    int n;
+    __device__ bool live(int v) const { return d.hc[v].x != -1; }
+    __device__ int degree(int v) const { return d.deg[v]; }
+    __device__ int* core(int v) const { return &d.hc[v].x; }
+    __device__ void list(int v, long long& off, int& len) const {
+        off = d.off[v];
+        len = d.end[v];
     }
-    __syncthreads();
-    int pre = 0;
-    for (int i = 0; i < wib; i++) pre += S.wcnt[i];
-    for (int i = lane_id(); i < cnt; i += 32) P.F[S.wbase + pre + i] = S.buf[wib][i];
-    cnt = 0;
-}
-
-// Slots [s0, s1) of the list at offset o (s0 a multiple of 4) at level k:
-// one degree off every neighbour; a neighbour that reaches k leaves now and
-// goes to the warp's buffer.  Four slots per lane per step with one 16-byte
-// load (lists start 16-byte aligned, capacities are multiples of 4).
-// Warp-collective.
-__device__ __forceinline__ void peel_range(const DevGraph& g, const PeelParams& P, Ctl* C, long long o, int s0,
-                                           int s1, int k, int32_t* buf, int& cnt) {
-    const int lane = lane_id();
-    for (int base = s0; base < s1; base += 128) {
-        const int t0 = base + lane * 4;
-        int4 a = make_int4(HOLE, HOLE, HOLE, HOLE);
-        if (t0 < s1) a = __ldcs(reinterpret_cast<const int4*>(g.adj + o + t0));
-        const int w[4] = {a.x, t0 + 1 < s1 ? a.y : HOLE, t0 + 2 < s1 ? a.z : HOLE, t0 + 3 < s1 ? a.w : HOLE};
-        int r[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) r[q] = w[q] >= 0 ? atomicSub(&P.dcur[w[q]], 1) : 0;
-        int mine = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) mine += w[q] >= 0 && r[q] == k + 1;
-        if (!__any_sync(0xffffffffu, mine != 0)) continue;
-        int incl = mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += t;
-        }
-        int at = cnt + incl - mine;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (w[q] >= 0 && r[q] == k + 1) {
-                g.hc[w[q]].x = k;
-                buf[at++] = w[q];
-            }
-        }
-        cnt += __shfl_sync(0xffffffffu, incl, 31);
-        __syncwarp();
-        if (cnt > kPushFlush) flush_peeled(C, P, buf, cnt);
-    }
-}
-
-// The peel's grid barrier.  The contract of grid_sync (the last block to
-// arrive copies the live tails and phase counters into their snapshots and
-// zeroes the counters before it releases the others; false once an error
-// is recorded), with the ordering carried by the operations themselves: the
-// arrival is an acquire-release add, the release a release store that also
-// carries the error state, each waiter's poll an acquire load.  The peel
-// runs ~5 barrier-separated phases per level, so the barrier's critical
-// path (last arrival, snapshot, release, the waiters' next poll) is a large
-// part of its time.  The release word is (generation << 1) | error; the
-// launch zone is zeroed before every peel launch.
-__device__ __forceinline__ bool peel_sync(Ctl* c, unsigned int expect, unsigned long long limit_ns) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t;
-        asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], 1;" : "=l"(t) : "l"(&c->arrive) : "memory");
-        const unsigned long long gen = t / expect;
-        int ok = 1;
-        if (t % expect == expect - 1) {
-            for (int i = 0; i < kTails; i++) {
-                c->stail[i] = vload64(&c->tail[i]);
-                c->spc[i] = vload64(&c->pc[i]);
-                c->pc[i] = 0;
-            }
-            ok = vload32(&c->error) == 0;
-            const unsigned long long rel = ((gen + 1) << 1) | (ok ? 0ull : 1ull);
-            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&c->release), "l"(rel) : "memory");
-        } else {
-            const unsigned long long t0 = gtimer();
-            unsigned int spins = 0;
-            for (;;) {
-                const unsigned long long rel = ld_acquire64(&c->release);
-                if ((rel >> 1) >= gen + 1) {
-                    ok = (rel & 1ull) == 0;
-                    break;
-                }
-                if (vload32(&c->error)) {
-                    ok = 0;
-                    break;
-                }
-                if ((++spins & 63u) == 0 && gtimer() - t0 > limit_ns) {
-                    atomicCAS(&c->error, 0, E_BARRIER_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(32);
-            }
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
-// Phases of the peel timed at its barriers (block 0's view, into Ctl::ph):
-// the level scans, the sub-waves and the chunk phases.
-enum { PP_SCAN = 0, PP_WAVE = 1, PP_CHUNK = 2 };
-struct PeelClock {
-    Ctl* c;
-    unsigned long long t;
-    bool on;
-    __device__ bool sync(const PeelParams& P, int phase) {
-        const bool ok = peel_sync(c, P.expect, P.limit_ns);
-        if (on) {
-            const unsigned long long now = gtimer();
-            c->ph[phase] += now - t;
-            c->st[ST_BARRIERS] += 1;
-            t = now;
-        }
-        return ok;
+    __device__ int quads(long long, int len) const { return (len + 3) >> 2; }
+    __device__ int4 quad(long long off, int len, int j) const {
+        int4 a = __ldcs(reinterpret_cast<const int4*>(d.adj + off + 4ll * j));
+        if (4 * j + 1 >= len) a.y = HOLE;
+        if (4 * j + 2 >= len) a.z = HOLE;
+        if (4 * j + 3 >= len) a.w = HOLE;
+        return a;
     }
 };
 
-__global__ void __launch_bounds__(kPeelThreads) peel_kernel(PeelParams P) {
-    Ctl* C = P.ctl;
-    const DevGraph g = P.g;
+__global__ void __launch_bounds__(kPeelThreads, 1) peel_kernel(PeelParams P) {
     __shared__ PeelShared S;
-    const int lane = lane_id();
-    const int wib = threadIdx.x >> 5;
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nthr = (long long)gridDim.x * blockDim.x;
-    const long long gwarp = gtid >> 5, nwarps = nthr >> 5;
-    int32_t* buf = S.buf[wib];
-    int cnt = 0;
-    PeelClock clk{C, gtimer(), blockIdx.x == 0 && threadIdx.x == 0};
-    // live vertices start unpeeled with their live degree (compacted into
-    // the remaining list a tile at a time, like the level scans below)
-    for (long long t0 = (long long)blockIdx.x * kScanTile; t0 < g.n; t0 += (long long)gridDim.x * kScanTile) {
-        if (threadIdx.x == 0) S.nkeep = 0;
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const long long v = t0 + q * kPeelThreads + threadIdx.x;
-            bool live = false;
-            if (v < g.n) {
-                live = g.hc[v].x != -1;
-                if (live) {
-                    P.dcur[v] = g.deg[v];
-                    g.hc[v].x = UNPEELED;
-                }
-            }
-            const unsigned lb = __ballot_sync(0xffffffffu, live);
-            int kp = 0;
-            if (lane == 0 && lb) kp = atomicAdd(&S.nkeep, __popc(lb));
-            kp = __shfl_sync(0xffffffffu, kp, 0);
-            if (live) S.keep[kp + __popc(lb & ((1u << lane) - 1))] = (int32_t)v;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) S.kbase = S.nkeep ? atomicAdd(&C->pc[1], (unsigned long long)S.nkeep) : 0;
-        __syncthreads();
-        for (int j = threadIdx.x; j < S.nkeep; j += kPeelThreads) P.L0[S.kbase + j] = S.keep[j];
-        __syncthreads();
-    }
-    if (!clk.sync(P, PP_SCAN)) return;
-    unsigned long long nl = vload64(&C->spc[1]);
-    int32_t* Lc = P.L0;
-    int32_t* Ln = P.L1;
-    int k = 0;
-    unsigned long long ft = 0;
-    long long levels = 0;
-    long long slots = 0;   // adjacency slots this warp scanned (algorithmic-byte counters)
-    while (nl > 0) {
-        // scan the remaining list, one tile per block at a time: degree k
-        // leaves now, above k stays, below k left at an earlier level
-        if (blockIdx.x == 0 && threadIdx.x == 0) C->st[ST_VISITED] += nl;
-        const unsigned long long f0 = ft;
-        for (long long t0 = (long long)blockIdx.x * kScanTile; t0 < (long long)nl;
-             t0 += (long long)gridDim.x * kScanTile) {
-            if (threadIdx.x == 0) {
-                S.nkeep = 0;
-                S.npeel = 0;
-                S.mx = 0;
-            }
-            __syncthreads();
-            int mx = 0;
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const long long i = t0 + q * kPeelThreads + threadIdx.x;
-                bool peel = false, keep = false;
-                int v = 0;
-                if (i < (long long)nl) {
-                    v = Lc[i];
-                    const int d = P.dcur[v];
-                    if (d == k) {
-                        g.hc[v].x = k;
-                        peel = true;
-                    } else if (d > k) {
-                        keep = true;
-                        mx = max(mx, 0x7FFFFFFF - d);
-                    }
-                }
-                const unsigned kb = __ballot_sync(0xffffffffu, keep), pb = __ballot_sync(0xffffffffu, peel);
-                int kp = 0, pp = 0;
-                if (lane == 0) {
-                    if (kb) kp = atomicAdd(&S.nkeep, __popc(kb));
-                    if (pb) pp = atomicAdd(&S.npeel, __popc(pb));
-                }
-                kp = __shfl_sync(0xffffffffu, kp, 0);
-                pp = __shfl_sync(0xffffffffu, pp, 0);
-                const unsigned below = (1u << lane) - 1;
-                if (keep) S.keep[kp + __popc(kb & below)] = v;
-                if (peel) S.peel[pp + __popc(pb & below)] = v;
-            }
-            for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            if (lane == 0 && mx) atomicMax(&S.mx, mx);
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                S.kbase = S.nkeep ? atomicAdd(&C->pc[1], (unsigned long long)S.nkeep) : 0;
-                S.pbase = S.npeel ? atomicAdd(&C->tail[0], (unsigned long long)S.npeel) : 0;
-                if (S.mx) atomicMax(&C->pc[3], (unsigned long long)S.mx);
-            }
-            __syncthreads();
-            for (int j = threadIdx.x; j < S.nkeep; j += kPeelThreads) Ln[S.kbase + j] = S.keep[j];
-            for (int j = threadIdx.x; j < S.npeel; j += kPeelThreads) P.F[S.pbase + j] = S.peel[j];
-            __syncthreads();
-        }
-        if (!clk.sync(P, PP_SCAN)) return;
-        unsigned long long fhi = vload64(&C->stail[0]);
-        unsigned long long nln = vload64(&C->spc[1]);
-        unsigned long long smx = vload64(&C->spc[3]);
-        int32_t* t = Lc;
-        Lc = Ln;
-        Ln = t;
-        nl = nln;
-        if (fhi == f0) {
-            if (nl == 0) break;
-            k = 0x7FFFFFFF - (int)smx;   // jump to the smallest remaining degree
-            continue;
-        }
-        // sub-waves at level k.  A peeled neighbour needs no test: its
-        // working degree is at most k when it leaves and only falls after,
-        // so a decrement can bring exactly k + 1 down to k only for a
-        // vertex still in the graph.
-        unsigned long long lo = f0, hi = fhi;
-        while (hi > lo) {
-            const unsigned long long cnt_f = hi - lo;
-            for (unsigned long long j = (unsigned long long)gwarp; j < cnt_f; j += (unsigned long long)nwarps) {
-                const int v = P.F[lo + j];
-                const long long o = g.off[v];
-                const int len = g.end[v];
-                slots += len;
-                if (len >= kPeelBig) {
-                    // chunk tasks (vertex, chunk), run by every warp after the barrier
-                    const int nch = (len + kPeelChunk - 1) / kPeelChunk;
-                    unsigned long long tb = 0;
-                    if (lane == 0) tb = atomicAdd(&C->pc[3], (unsigned long long)nch);
-                    tb = __shfl_sync(0xffffffffu, tb, 0);
-                    const bool fits = tb + nch <= P.chunk_cap;
-                    for (int c = lane; c < nch; c += 32) {
-                        if (tb + c >= P.chunk_cap) break;
-                        P.chunks[tb + c] = fits ? (((unsigned long long)(uint32_t)v << 32) | (uint32_t)c)
-                                                : kPeelNoTask;
-                    }
-                    if (fits) continue;
-                }
-                peel_range(g, P, C, o, 0, len, k, buf, cnt);
-            }
-            block_flush_peeled(C, P, S, cnt);
-            if (!clk.sync(P, PP_WAVE)) return;
-            const unsigned long long nchunks = min(vload64(&C->spc[3]), P.chunk_cap);
-            if (nchunks > 0) {
-                for (unsigned long long c = (unsigned long long)gwarp; c < nchunks; c += (unsigned long long)nwarps) {
-                    const unsigned long long task = P.chunks[c];
-                    if (task == kPeelNoTask) continue;
-                    const int v = (int)(task >> 32);
-                    const int s0 = (int)(task & 0xFFFFFFFFu) * kPeelChunk;
-                    peel_range(g, P, C, g.off[v], s0, min(g.end[v], s0 + kPeelChunk), k, buf, cnt);
-                }
-                block_flush_peeled(C, P, S, cnt);
-                if (!clk.sync(P, PP_CHUNK)) return;
-            }
-            if (blockIdx.x == 0 && threadIdx.x == 0) C->st[ST_WAVES]++;
-            lo = hi;
-            hi = vload64(&C->stail[0]);
-        }
-        ft = hi;
-        k++;
-        levels++;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) C->st[ST_LEVELS] = (unsigned long long)levels;
-    if (lane == 0 && slots) atomicAdd(&C->st[ST_VISSLOTS], (unsigned long long)slots);
+    const PeelStore g{P.g, P.g.n};
+    const PeelWork W{P.ctl, P.dcur, P.list, P.far, P.chunks, P.chunk_cap, gridDim.x, P.limit_ns};
+    peel_graph(g, W, S);
 }
 
-// The peel always runs kPeelThreads-thread blocks (its tiles and per-warp
-// buffers are laid out for them); `threads` is ignored.
-int peel_blocks_per_sm(int threads) {
-    (void)threads;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, peel_kernel, kPeelThreads, 0) != cudaSuccess) return 0;
-    return nb;
-}
-
-cudaError_t launch_peel(const PeelParams& p, int blocks, int threads, cudaStream_t s) {
-    (void)threads;
+// Cooperative: at most one block per SM, which the grid barrier needs resident.
+cudaError_t launch_peel(const PeelParams& p, int blocks, cudaStream_t s) {
     PeelParams q = p;
     void* args[] = {&q};
     return cudaLaunchCooperativeKernel((const void*)peel_kernel, dim3(blocks), dim3(kPeelThreads), args, 0, s);
