@@ -81,9 +81,9 @@ typedef struct cm_options {
     int32_t block_mode_leave; /* single block -> grid after an iteration touching more (8192) */
     int32_t hub_slots;      /* grid mode: a vertex with at least this many adjacency slots is scanned by
                                all warps in chunks of 512 (1024; negative = never) */
-    int32_t block_slots;    /* grid mode, insert: a vertex with at least this many slots (below hub_slots)
-                               is scanned by a whole block instead of one warp (4096) */
-    int32_t block_slots_delete; /* the same for delete calls (1024) */
+    int32_t block_slots;    /* grid mode, insert: outside the search, a vertex with at least this many slots
+                               is scanned by a whole block instead of one warp (4096, the least that counts) */
+    int32_t block_slots_delete; /* the same for delete calls (values below 4096 count as 4096) */
     int32_t task_claim;     /* grid mode: multiple of its fair share of the waiting search tasks that a warp
                                claims at once (1..8, default 1) */
     int32_t select_order;   /* order of the greedy superior-edge-set selection (Section IV,

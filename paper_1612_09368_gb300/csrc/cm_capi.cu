@@ -22,7 +22,7 @@
 using namespace cm;
 
 static thread_local std::string g_create_err = "no error";
-constexpr int kGridThreadsHost = 512;   // threads per block of both maintenance kernels
+constexpr int kGridThreadsHost = 384;   // threads per block of the grid-mode kernels (kGridThreads)
 
 struct cm_graph {
     cm_options opt;
@@ -70,7 +70,7 @@ struct cm_graph {
     HubItem* HQ = nullptr;
     unsigned long long* TQ = nullptr;   // grid-mode task queue (TASK_EMPTY = all ones when free)
     unsigned long long tq_size = 0;
-    // candidate records of the grid-mode search (cm_search.cuh): per vertex
+    // records of the grid-mode search (cm_search.cuh): per vertex
     // a stamped position in the arena
     unsigned long long* rec = nullptr;
     size_t rec_size = 0;
@@ -298,13 +298,13 @@ static int ensure_tasks(cm_graph* h) {
     return CM_OK;
 }
 
-// Candidate records of the search: a word per vertex, and an arena of a
-// quarter of the adjacency pool for one iteration's records (a search that
-// fills it scans the lists of the vertices left out again).
+// Records of the search: a word per vertex, and an arena of two thirds of the
+// adjacency pool's bytes for a launch's records (a search that fills it scans
+// the lists of the vertices left out).
 static int ensure_records(cm_graph* h) {
     if (h->rec_size < (size_t)h->ncap) {
         unsigned long long* q = (unsigned long long*)dalloc(h, (size_t)h->ncap * 8);
-        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the candidate records");
+        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the search records");
         CK(h, cudaMemsetAsync(q, 0, (size_t)h->ncap * 8, h->stream));   // stamp 0 names no iteration
         if (h->rec) {
             CK(h, cudaStreamSynchronize(h->stream));
@@ -313,10 +313,10 @@ static int ensure_records(cm_graph* h) {
         h->rec = q;
         h->rec_size = (size_t)h->ncap;
     }
-    const unsigned long long quads = (unsigned long long)h->g.adj_cap / 16 + 1024;
+    const unsigned long long quads = (unsigned long long)h->g.adj_cap / 6 + 1024;
     if (h->arena_quads < quads) {
         int32_t* q = (int32_t*)dalloc(h, (size_t)quads * 16);
-        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the candidate arena");
+        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the record arena");
         if (h->arena) {
             CK(h, cudaStreamSynchronize(h->stream));
             dfree(h, h->arena, (size_t)h->arena_quads * 16);
@@ -365,8 +365,12 @@ static int ensure_batch(cm_graph* h, long long k) {
 
 // ------------------------------------------------------------------ launch geometry
 // The maintenance kernel fills max_sms SMs (all by default) with as many
-// blocks as stay resident.  A small batch gets fewer blocks: grid barriers then
-// cost less, and there is not enough work for the whole GPU anyway.
+// blocks as stay resident.  A small batch on a small graph gets one block per
+// SM: grid barriers then cost less, and there is not enough work for more.  A
+// small batch on a large graph needs them all: a few edges can search a dense
+// shell of it (R-MAT scale 24, 10^3 degree-proportional edges: 12.3 -> 9.7 ms
+// with all blocks), so the bound follows the graph too, one thread per 32
+// list entries.
 static void persistent_geometry(cm_graph* h, long long work, int* blocks, int* threads) {
     const int t = kGridThreadsHost;
     int occ = maintain_blocks_per_sm(t);
@@ -375,7 +379,8 @@ static void persistent_geometry(cm_graph* h, long long work, int* blocks, int* t
     int sms = h->opt.max_sms > 0 && h->opt.max_sms < h->num_sms ? h->opt.max_sms : h->num_sms;
     long long b = (long long)sms * bps;
     if (h->opt.blocks_per_sm <= 0) {
-        long long want = (work * 64 + t - 1) / t;
+        const long long by_graph = 2 * (long long)h->m / 32;
+        long long want = ((work * 64 > by_graph ? work * 64 : by_graph) + t - 1) / t;
         if (want < sms) want = sms;
         if (want < b) b = want;
     }
@@ -877,7 +882,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
                 return set_err(h, CM_ERR_LIMIT, "maintenance did not finish within %d launch pairs", pass);
             }
             if (want_grid) LAUNCH(h, launch_maintain(p, blocks, threads, h->stream));
-            LAUNCH(h, launch_maintain_block(p, 1024, h->stream));
+            LAUNCH(h, launch_maintain_block(p, h->stream));
             if ((rc = rd_ctl(h))) return rc;
             if (check_each && !c.error) {
                 cm_check_report r{};
@@ -1503,7 +1508,7 @@ static cudaError_t capture_loop(cm_step* s, int op) {
     p.use_cond = 1;
     p.cond = (unsigned long long)hc;
     cudaError_t e1 = launch_maintain(p, blocks, threads, s->cs2);
-    cudaError_t e2 = e1 == cudaSuccess ? launch_maintain_block(p, kGridThreadsHost, s->cs2) : e1;
+    cudaError_t e2 = e1 == cudaSuccess ? launch_maintain_block(p, s->cs2) : e1;
     cudaGraph_t out = nullptr;
     cudaError_t e3 = cudaStreamEndCapture(s->cs2, &out);
     return e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3;

@@ -95,22 +95,23 @@ constexpr int kTails = 4;
 // HUB_EVICT_INS / HUB_EVICT_DEL (eviction scans), HUB_EXPAND (visit the
 // frontier neighbours of a hub whose support stayed above k).
 // HUB_FRONT_SPEC: as HUB_FRONT, but each chunk also visits its candidates
-// at once (see expand_early) and records them, so no HUB_EXPAND round
-// follows.  HUB_EVICT_REC: eviction of the recorded candidates (off and len
-// are those of the record).
+// at once (see expand_early) and leaves a record of the vertex's core-k
+// neighbours, so no HUB_EXPAND round follows.  HUB_FRONT_REC, HUB_EVICT_REC:
+// the same from the record (off and len are the record's, in the arena).
 enum {
-    HUB_FRONT = 0, HUB_EVICT_INS = 1, HUB_EVICT_DEL = 2, HUB_EXPAND = 3, HUB_FRONT_SPEC = 4, HUB_EVICT_REC = 5
+    HUB_FRONT = 0, HUB_EVICT_INS = 1, HUB_EVICT_DEL = 2, HUB_EXPAND = 3, HUB_FRONT_SPEC = 4, HUB_EVICT_REC = 5,
+    HUB_FRONT_REC = 6
 };
 struct __align__(16) HubItem {
     long long off;                 // adjacency offset
     int32_t v, kind, k, len;
     int32_t nch;                   // chunks
-    int32_t acc;                   // partial-sum accumulator (HUB_FRONT)
+    int32_t acc;                   // partial-sum accumulator (HUB_FRONT*); HUB_EVICT_REC: 1 if its marks are old
     uint32_t done;                 // chunks finished
-    int32_t rcur;                  // recorded candidates so far
-    unsigned long long rquad;      // their record's first arena quad
+    int32_t rcur;                  // ids in its record so far
+    unsigned long long rquad;      // the record's first arena quad
     int32_t rcap;                  // ... and room (0: none)
-    int32_t pad;
+    int32_t ncand;                 // candidates among the list so far
 };
 constexpr int kChunk = 512;                 // slots per chunk: one scan step of a warp
 constexpr unsigned long long kHubRing = 1ull << 20;
@@ -150,7 +151,8 @@ struct __align__(128) Ctl {
     alignas(128) unsigned long long task_done;  // tasks finished
     alignas(128) unsigned long long hub_created;    // hub items of the current search
     unsigned long long hub_finished;
-    alignas(128) unsigned long long rec_top;    // next free quad of the candidate arena
+    alignas(128) unsigned long long quiet;      // iteration whose search is known to be quiescent
+    alignas(128) unsigned long long rec_top;    // next free quad of the record arena
     alignas(128) Resume rs;
 };
 

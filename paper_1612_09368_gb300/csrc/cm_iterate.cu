@@ -59,6 +59,8 @@
 // dynamically); a vertex with at least P.block_len adjacency slots (256 in
 // single-block mode) is deferred
 // and then processed by the whole block of the warp that fetched it.
+#include <type_traits>
+
 #include "cm_common.cuh"
 #include "cm_launch.h"
 #include "cm_search.cuh"
@@ -67,10 +69,31 @@
 namespace cm {
 
 constexpr int kBlockThreads = 512;    // single-block mode
-constexpr int kGridThreads = 512;     // grid mode, per block
+// Grid mode, per block, two blocks per SM: 80 registers a thread.  The search
+// needs about 90; at 64 (512 threads) the spills, which are written through to
+// L2, cost more than the warps gain.  512 / 448 / 384 / 320 threads, one pass
+// of inserts and deletes: R-MAT scale 20 with 10^4 edges 3.4 / 3.2 / 3.0 / 3.1
+// ms, Erdos-Renyi 2*10^6 with 10^4 4.2 / 4.1 / 4.0 / 3.9 ms, R-MAT scale 24
+// with 10^3 degree-proportional - / 10.3 / 9.7 / 10.4 ms.
+constexpr int kGridThreads = 384;
 static_assert(kGridThreads / 32 == kGridWarps, "one search buffer per grid-mode warp");
 constexpr int kMaxBig = 64;
 constexpr int kBlockLenSingle = 256;   // single-block mode: the block scans lists from this size
+// Grid mode: never below this, whatever the options say.  A warp walks 512
+// slots a step, so a block on a shorter list leaves most of its warps idle
+// (10^6 degree-proportional deletes on R-MAT scale 24, 1024 -> 4096: 30.3 ->
+// 26.9 ms).
+constexpr int kBlockLenGrid = 4096;
+
+// The iteration loop's state while a grid-wide search runs.
+struct LoopState {
+    unsigned long long nrem, nrem_next, vq0, eq0, cq0, vq_t, eq_t, cq_t;
+    REdge *Rc, *Rn;
+    unsigned long long t_last;
+    long long remsum, iters0;
+    uint32_t e, e0;
+    int iters, rounds, waves;
+};
 
 template <int MODE>
 struct Barrier {
@@ -97,8 +120,8 @@ struct Barrier {
 // dynamically (counter *ctr, zeroed at every barrier), so a phase with no
 // more vertices than warps touches no shared counter, and a larger one does
 // not start with every warp of the grid at the same counter.  A vertex
-// with at least P.block_len slots (kBlockLenSingle in single-block mode) is
-// deferred by the warp that fetched it and then processed by that warp's
+// with at least P.block_len slots (kBlockLenGrid at least; kBlockLenSingle in
+// single-block mode) is deferred by the warp that fetched it and then processed by that warp's
 // whole block, so a long list does not hold a wave on one warp.  Every
 // thread of the launch must call it.
 template <int MODE, class Body>
@@ -118,7 +141,7 @@ __device__ __forceinline__ void for_each_vertex(const DevGraph& g, const Maintai
         if (j >= cnt) break;
         const int v = ring[(lo + j) & qm];
         int defer = 0;
-        if (lane == 0 && g.end[v] >= (MODE == 0 ? P.block_len : kBlockLenSingle)) {
+        if (lane == 0 && g.end[v] >= (MODE == 0 ? max(P.block_len, kBlockLenGrid) : kBlockLenSingle)) {
             int s = atomicAdd(&s_nbig, 1);
             if (s < kMaxBig) {
                 s_big[s] = v;
@@ -249,7 +272,9 @@ __device__ __forceinline__ void loop_control(const MaintainParams& P, Ctl* C) {
     cudaGraphSetConditional((cudaGraphConditionalHandle)P.cond, (!err && !done) ? 1u : 0u);
 }
 
-template <int MODE>
+// One kernel per mode and operation (OP 0 insert, 1 delete): each carries one
+// search only, which keeps its registers and instructions within bounds.
+template <int MODE, int OP>
 __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE == 0 ? 2 : 1)
     maintain_kernel(MaintainParams P) {
     Ctl* C = P.ctl;
@@ -261,11 +286,15 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         if (MODE == 1) loop_control(P, C);
         return;
     }
-    if (MODE == 0) {   // shared memory starts undefined: no search is quiescent yet
+    const int lane = lane_id();
+    if (MODE == 0) {   // shared memory starts undefined: no search is quiescent yet, no warp holds arena room
         if (threadIdx.x == 0) s_quiet = ~0u;
+        WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
+        if (lane == 0) B.slab = B.slab_end = 0;
+        if (lane < 7) B.st[lane] = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) C->rec_top = 0;
         __syncthreads();
     }
-    const int lane = lane_id();
     const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     const unsigned long long qm = P.qmask;
@@ -276,7 +305,8 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
     REdge* Rn = rsel0 ? P.R0 : P.R1;
     unsigned long long nrem = vload64(&C->rs.nrem);
     uint32_t e = *(volatile uint32_t*)&C->rs.epoch;
-    const long long iters0 = *(volatile long long*)&C->rs.iters;
+    uint32_t e0 = e;         // records of this launch carry stamps from here on
+    long long iters0 = *(volatile long long*)&C->rs.iters;
     unsigned long long vq_t = vload64(&C->tail[0]), eq_t = vload64(&C->tail[1]), cq_t = vload64(&C->tail[2]);
     // grid mode: the task queue starts empty for every search
     auto reset_tasks = [&]() {
@@ -286,7 +316,6 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             C->task_done = 0;
             C->hub_created = 0;
             C->hub_finished = 0;
-            C->rec_top = 0;
         }
     };
     LocalStats ls;
@@ -316,8 +345,53 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
     uint32_t fx_e = 0;
     // a call whose ingest kept no edge (its count read on the device) is done at once
     int next_want = MODE, finished = (!mid && nrem == 0) ? 1 : 0;
-    const int32_t* FXQ = P.op == 0 ? P.CQ : P.EQ;
-    auto fixup_body = [&](int v, auto grp) { fixup_vertex<decltype(grp)>(g, v, fx_e, P.op, ls); };
+    const int32_t* FXQ = OP == 0 ? P.CQ : P.EQ;
+    auto fixup_body = [&](int v, auto grp) {
+        if constexpr (MODE == 0)
+            fixup_wide<OP, decltype(grp)>(g, P, reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5], v, fx_e, e0,
+                                          nrem > 0);
+        else
+            fixup_vertex<decltype(grp)>(g, v, fx_e, OP, ls);
+    };
+
+    // The grid-wide search, with the loop's state parked in shared memory
+    // meanwhile (every thread holds the same values): see flush_stats.
+    [[maybe_unused]] auto search = [&](auto del) {
+        if constexpr (MODE == 0) {
+            WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
+            flush_stats(B, ls);
+            __shared__ LoopState S;
+            __syncthreads();   // the last reader of S is done
+            if (threadIdx.x == 0) {
+                S = LoopState{nrem, nrem_next, vq0, eq0, cq0, vq_t, eq_t, cq_t, Rc, Rn, sync.t_last, remsum, iters0,
+                              e, e0, iters, rounds, waves};
+                s_search_t0 = gtimer();
+            }
+            __syncthreads();
+            const bool fine = async_search<decltype(del)::value>(g, C, P, S.e, S.e0, OP == 0 && S.nrem_next > 0);
+            nrem = S.nrem;
+            nrem_next = S.nrem_next;
+            vq0 = S.vq0;
+            eq0 = S.eq0;
+            cq0 = S.cq0;
+            vq_t = S.vq_t;
+            eq_t = S.eq_t;
+            cq_t = S.cq_t;
+            Rc = S.Rc;
+            Rn = S.Rn;
+            sync.t_last = S.t_last;
+            remsum = S.remsum;
+            iters0 = S.iters0;
+            e = S.e;
+            e0 = S.e0;
+            iters = S.iters;
+            rounds = S.rounds;
+            waves = S.waves;
+            return fine;
+        } else {
+            return true;
+        }
+    };
 
     while (mid || nrem > 0) {
       if (!mid) {
@@ -337,13 +411,13 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             if (MODE == 0 && r == 0) reset_tasks();   // nobody pushes tasks before APPLY
             for (long long base = gwarp * 32; base < (long long)nrem; base += nwarps * 32) {
                 long long i = base + lane;
-                if (i < (long long)nrem) claim_edge(g, Rc, i, r, e, P.sel_key != 0, P.op == 0);
+                if (i < (long long)nrem) claim_edge(g, Rc, i, r, e, P.sel_key != 0, OP == 0);
             }
             if (!(ok = sync(PH_CLAIM))) break;
             int lost = 0;
             for (long long base = gwarp * 32; base < (long long)nrem; base += nwarps * 32) {
                 long long i = base + lane;
-                if (i < (long long)nrem) lost += check_edge(g, Rc, i, r, e, ls.sel, P.sel_key != 0, P.op == 0);
+                if (i < (long long)nrem) lost += check_edge(g, Rc, i, r, e, ls.sel, P.sel_key != 0, OP == 0);
             }
             lost = warp_sum(lost);
             if (lane == 0 && lost) atomicAdd(&C->pc[0], (unsigned long long)lost);
@@ -367,7 +441,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                 E = Rc[i];
                 int k = 0; bool clo = false, chi = false;
                 // only a selected edge or one that claimed in the final round needs its level
-                if ((E.flags & F_SEL) || (E.flags >> 2) == (uint32_t)r) edge_level(g, E, P.op == 0, k, clo, chi);
+                if ((E.flags & F_SEL) || (E.flags >> 2) == (uint32_t)r) edge_level(g, E, OP == 0, k, clo, chi);
                 if ((E.flags >> 2) == (uint32_t)r) {     // claimed in the final round
                     unsigned long long* cb = ((r - 1) & 1) ? g.claim1 : g.claim0;
                     if (clo) cb[E.lo] = CLAIM_FREE;
@@ -375,7 +449,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                 }
                 sel = (E.flags & F_SEL) != 0;
                 if (sel) {
-                    if (P.op == 0) {
+                    if constexpr (OP == 0) {
                         int pu = atomicAdd(&g.end[E.lo], 1), pv = atomicAdd(&g.end[E.hi], 1);
                         if (pu < g.cap[E.lo] && pv < g.cap[E.hi]) {
                             g.adj[g.off[E.lo] + pu] = E.hi;
@@ -390,6 +464,10 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                         // a constrained endpoint's SD rises; with SD > k it roots the search
                         // (one selected edge per constrained endpoint and level: this is the
                         // only SD change of the endpoint in APPLY, so its key bit follows it)
+                        if (MODE == 0) {
+                            if (clo) rec_link(P, e0, E.lo, k, E.hi, !chi);
+                            if (chi) rec_link(P, e0, E.hi, k, E.lo, !clo);
+                        }
                         if (clo) {
                             const int sd = atomicAdd(&g.hc[E.lo].y, 1) + 1;
                             if (sd > k) atomicOr(&g.kc[E.lo], 1u);
@@ -427,8 +505,8 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             }
             warp_push_edge(&C->pc[1], Rn, valid && !sel, E);
             // roots: frontier (insert) or evicted (delete) constrained endpoints
-            push_vertex<MODE == 0>(C, P, s_lo, E.lo, P.op == 0 ? 0 : 1);
-            push_vertex<MODE == 0>(C, P, s_hi, E.hi, P.op == 0 ? 0 : 1);
+            push_vertex<MODE == 0>(C, P, s_lo, E.lo, OP == 0 ? 0 : 1);
+            push_vertex<MODE == 0>(C, P, s_hi, E.hi, OP == 0 ? 0 : 1);
         }
         if (!(ok = sync(PH_APPLY))) break;
         nrem_next = vload64(&C->spc[1]);
@@ -442,7 +520,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
       const bool resumed = mid;
       mid = false;
 
-        if (P.op == 0) {
+        if constexpr (OP == 0) {
             // -------------------------------------------- SEARCH (insert): frontier + evictions
             if constexpr (MODE == 0) {
                 if (resumed) {   // the single-block mode began this search
@@ -453,7 +531,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     if (!(ok = sync(PH_APPLY))) break;
                 }
                 waves++;
-                ok = async_search<false>(g, C, P, e, ls);
+                ok = search(std::false_type{});
                 if (!(ok = sync(PH_DISCOVER) && ok)) break;
                 fhi = vload64(&C->stail[0]);
                 ehi = vload64(&C->stail[1]);
@@ -516,7 +594,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     if (!(ok = sync(PH_APPLY))) break;
                 }
                 waves++;
-                ok = async_search<true>(g, C, P, e, ls);
+                ok = search(std::true_type{});
                 if (!(ok = sync(PH_EVICT) && ok)) break;
                 ehi = vload64(&C->stail[1]);
             } else {
@@ -544,7 +622,9 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         fx_e = e;
         // ------------------------------------------------ next iteration, or hand over
         const unsigned long long nsel = nrem - nrem_next;
-        const unsigned long long work = (vq_t - vq0) + (eq_t - eq0) + (cq_t - cq0) + nsel;
+        // (a grid-wide insertion logs no evictions: they are about as many as the visits)
+        const unsigned long long work = (vq_t - vq0) * (MODE == 0 && OP == 0 ? 2 : 1) + (eq_t - eq0) +
+                                        (cq_t - cq0) + nsel;
         REdge* t = Rc;
         Rc = Rn;
         Rn = t;
@@ -573,12 +653,12 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         ok = sync(PH_FIXUP);
     }
     // statistics: one atomic per warp
-    const uint32_t mine[7] = {ls.vis, ls.visl, ls.ev, ls.evl, ls.ch, ls.chl, ls.sel};
+    uint32_t tot[7] = {ls.vis, ls.visl, ls.ev, ls.evl, ls.ch, ls.chl, ls.sel};
     const int slot[7] = {ST_VISITED, ST_VISSLOTS, ST_EVICTED, ST_EVSLOTS, ST_CHANGED, ST_CHSLOTS, ST_SELECTED};
 #pragma unroll
     for (int i = 0; i < 7; i++) {
-        unsigned long long t = mine[i];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        unsigned long long t = __reduce_add_sync(0xffffffffu, tot[i]);
+        if (MODE == 0) t += reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5].st[i];
         if (lane == 0 && t) atomicAdd(&C->st[slot[i]], t);
     }
     if (leader) {
@@ -617,17 +697,24 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
     if (MODE == 1) loop_control(P, C);   // thread 0 is the leader: its writes above come first
 }
 
-// The search's buffers exceed the default 48 KB of shared memory per block.
-static cudaError_t allow_search_smem() {
-    return cudaFuncSetAttribute(maintain_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSearchSmem);
+static const void* maintain_kernel(int mode, int op) {
+    return mode == 0 ? (op == 0 ? (const void*)maintain_kernel<0, 0> : (const void*)maintain_kernel<0, 1>)
+                     : (op == 0 ? (const void*)maintain_kernel<1, 0> : (const void*)maintain_kernel<1, 1>);
 }
 
+// Resident blocks per SM of the grid-mode kernels (both operations).  Their
+// search buffers exceed the default 48 KB of shared memory per block.
 int maintain_blocks_per_sm(int threads) {
-    int nb = 0;
-    if (allow_search_smem() != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, maintain_kernel<0>, threads, kSearchSmem) != cudaSuccess)
-        return 0;
-    return nb;
+    int least = 0;
+    for (int op = 0; op < 2; op++) {
+        const void* f = maintain_kernel(0, op);
+        int nb = 0;
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSearchSmem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, threads, kSearchSmem) != cudaSuccess)
+            return 0;
+        least = op == 0 || nb < least ? nb : least;
+    }
+    return least;
 }
 
 // Cooperative (co-resident blocks, which the grid barrier needs); the
@@ -643,17 +730,15 @@ cudaError_t launch_maintain(const MaintainParams& p, int blocks, int threads, cu
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, maintain_kernel<0>, p);
+    MaintainParams q = p;
+    void* args[] = {&q};
+    return cudaLaunchKernelExC(&cfg, maintain_kernel(0, p.op), args);
 }
 
-const void* maintain_kernel_symbol(int mode) {
-    return mode == 0 ? (const void*)maintain_kernel<0> : (const void*)maintain_kernel<1>;
-}
-
-cudaError_t launch_maintain_block(const MaintainParams& p, int threads, cudaStream_t s) {
-    (void)threads;
-    maintain_kernel<1><<<1, kBlockThreads, 0, s>>>(p);
-    return cudaGetLastError();
+cudaError_t launch_maintain_block(const MaintainParams& p, cudaStream_t s) {
+    MaintainParams q = p;
+    void* args[] = {&q};
+    return cudaLaunchKernel(maintain_kernel(1, p.op), dim3(1), dim3(kBlockThreads), args, 0, s);
 }
 
 }  // namespace cm

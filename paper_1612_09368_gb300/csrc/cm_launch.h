@@ -37,7 +37,7 @@ struct MaintainParams {
     HubItem* HQ;              // hub items of the current search (ring of kHubRing)
     unsigned long long* TQ;   // grid-mode task queue (ring, TASK_EMPTY when free)
     unsigned long long tqmask;
-    unsigned long long* rec;  // per vertex: where its candidates are recorded in `arena` (stamped, see cm_search.cuh)
+    unsigned long long* rec;  // per vertex: where its record is in `arena` (stamped, see cm_search.cuh)
     int32_t* arena;
     unsigned long long arena_quads;
     uint32_t slab_quads;      // arena quads a warp takes at a time
@@ -85,9 +85,7 @@ cudaError_t phase_maintain(Ctl* c, StepLog* log, int phase, cudaStream_t s);
 cudaError_t phase_end(Ctl* c, StepLog* log, int phase, cudaStream_t s);
 cudaError_t apply_structure(const REdge* R, long long n, int op, DevGraph g, Ctl* c, cudaStream_t s);
 cudaError_t launch_maintain(const MaintainParams& p, int blocks, int threads, cudaStream_t s);
-cudaError_t launch_maintain_block(const MaintainParams& p, int threads, cudaStream_t s);
-// kernel symbols of the two execution modes, for graph capture
-const void* maintain_kernel_symbol(int mode);
+cudaError_t launch_maintain_block(const MaintainParams& p, cudaStream_t s);
 int maintain_blocks_per_sm(int threads);
 
 // ---- store / peel (cm_store.cu)

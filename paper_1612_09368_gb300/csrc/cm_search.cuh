@@ -21,15 +21,19 @@
 //     are few; they are compacted into a per-warp shared buffer, and their
 //     words and atomics are then handled 128 at a time, every lane busy.
 //   * tasks are taken 32 at a time, one per lane.  The lists of those with
-//     at most 128 slots are walked together, quad by quad (a quad is four
+//     at most 256 slots are walked together, quad by quad (a quad is four
 //     slots, one 16-byte load), up to 128 quads a window: lane l of a
 //     window's load takes quad l whoever owns it.  (With one warp per vertex
 //     a vertex of 9 slots used three lanes of 32 and cost a queue hand-off.)
 //   * a frontier vertex whose support stays at or below k is evicted by the
 //     task that found it out, from the candidates it still holds.
-//   * a longer list whose vertex survives leaves its candidates behind (an
-//     arena in device memory): if the vertex is evicted later, its eviction
-//     reads those few ids instead of the whole list and its keys.
+//   * the scan of a longer list leaves a record behind (an arena in device
+//     memory): the neighbours of core k and how many are above, a tenth to a
+//     quarter of the list.  The vertex is then walked from its record: when it
+//     is evicted later in the same search, and in the following iterations of
+//     the launch for as long as its core stays k (an insertion only raises
+//     cores, so the neighbours counted above stay above; edges and neighbours
+//     that join the level are appended, see rec_link).
 //
 // Measured search time (GB300, one warp per vertex and 128-slot steps -> this
 // layout): Erdos-Renyi, 2*10^6 vertices of degree 8, 10^4 uniform inserts 6.5
@@ -41,15 +45,15 @@
 //
 // A vertex with at least P.hub_len slots becomes a hub item instead, whose
 // list is split into kChunk-slot chunk tasks that any warp may take:
-//   HUB_FRONT / HUB_FRONT_SPEC: each chunk adds its share of CSD to the
-//     item; the warp that finishes the last chunk adds the sum to the
+//   HUB_FRONT / HUB_FRONT_SPEC / HUB_FRONT_REC: each chunk adds its share of
+//     CSD to the item; the warp that finishes the last chunk adds the sum to the
 //     support word at once (setting the processed flag, as a whole-list
 //     scan would) and either queues an expansion item (support > k; the
-//     SPEC chunks have visited their candidates already) or evicts the
-//     vertex;
+//     SPEC and REC chunks have visited their candidates already) or evicts
+//     the vertex;
 //   HUB_EXPAND: each chunk visits its share of the core-k neighbours;
 //   HUB_EVICT_INS / HUB_EVICT_DEL / HUB_EVICT_REC: each chunk evicts its
-//     share (REC: of the recorded candidates); the last one lowers the core
+//     share (REC: of the record); the last one lowers the core
 //     (delete) and counts the vertex.
 // The support word tolerates the delay: decrements from evicted neighbours
 // land before or after the CSD sum in any order, and a processed hub whose
@@ -61,55 +65,124 @@
 
 namespace cm {
 
-constexpr int kGridWarps = 16;    // warps per grid-mode block
+constexpr int kGridWarps = 12;    // warps per grid-mode block
 constexpr int kWindow = 512;      // slots of a scan step
-constexpr int kCand = 1024;       // candidates a warp holds: every list below the default hub_len fits
-constexpr int kShort = 128;       // lists up to this many slots are walked together
+// Lists up to this many slots are walked together (and not recorded).  64 /
+// 128 / 256 / 512: the captured step of 64 Barabasi-Albert graphs 51 / 45 /
+// 42 / 41 ms, R-MAT scale 20 with 10^4 edges 3.2 / 3.1 / 2.8 / 2.9 ms.
+constexpr int kShort = 256;
 
 // Per-warp scratch of the search (dynamic shared memory).
 struct WarpBuf {
-    int32_t id[kCand];                // candidates
+    int32_t id[kWindow];              // a window's candidates, and from the end its other core-k neighbours
     unsigned long long kept[32];      // tasks the warp keeps for itself
+    unsigned long long rec_q[32];     // records made but not published
+    int32_t rec_v[32];
+    unsigned long long slab, slab_end;   // arena quads the warp holds (for the whole launch)
+    uint32_t st[7];                   // statistics of the launch so far (N_*)
     int32_t csd[32];                  // CSD of the tasks walked together
     uint8_t own[kWindow];             // their candidates' tasks (lane numbers)
 };
 constexpr size_t kSearchSmem = sizeof(WarpBuf) * kGridWarps;
 extern __shared__ __align__(16) unsigned char s_search[];
 
+// Statistics kept per warp in shared memory: as registers they would be live
+// across the whole search, which is short of registers (a spilled register
+// is written through to L2: with the loop state and these spilled, local
+// memory took three times the requests of the lists and keys).
+enum { N_VIS = 0, N_VISL, N_EV, N_EVL, N_CH, N_CHL, N_SEL };
+__device__ __forceinline__ void note(WarpBuf& B, int what, uint32_t n) {   // one lane of the warp
+    B.st[what] += n;
+}
+__device__ __forceinline__ void flush_stats(WarpBuf& B, LocalStats& ls) {
+    const uint32_t mine[7] = {ls.vis, ls.visl, ls.ev, ls.evl, ls.ch, ls.chl, ls.sel};
+#pragma unroll
+    for (int i = 0; i < 7; i++) {
+        const uint32_t t = __reduce_add_sync(0xffffffffu, mine[i]);
+        if (lane_id() == 0) B.st[i] += t;
+    }
+    ls = LocalStats{};
+    __syncwarp();
+}
+
 __device__ __forceinline__ int vload32i(const int* p) { return *(const volatile int*)p; }
 
 // A vertex's record: the stamp of the iteration that wrote it (30 bits, as
-// in the per-iteration word) and the arena quad where its candidates start
-// (the first quad holds their count).  One 64-bit word, so a reader sees
-// both or neither; a stale stamp means "scan the list".
+// in the per-iteration word) and its first arena quad, in one 64-bit word,
+// so a reader sees both or neither.  The first quad is the header {count,
+// room, neighbours above k, k}; the ids follow, those that were candidates
+// (SD > k) with the sign bit set.  A record is fresh if it was made in this
+// launch (stamp >= e0, the launch's first iteration: the single-block mode
+// does not keep records up to date), and stands for the list at level k if
+// its k is that (-1: candidates only, for this iteration's evictions) and it
+// did not overflow (count > room).
+constexpr int32_t REC_CAND = (int32_t)0x80000000;
 __device__ __forceinline__ unsigned long long rec_word(unsigned long long quad, uint32_t e) {
     return (quad << 30) | (unsigned long long)(e & 0x3FFFFFFFu);
 }
-__device__ __forceinline__ bool rec_of(unsigned long long w, uint32_t e, unsigned long long& quad) {
-    quad = w >> 30;
-    return (uint32_t)(w & 0x3FFFFFFFull) == (e & 0x3FFFFFFFu);
+__device__ __forceinline__ uint32_t rec_stamp(unsigned long long w) { return (uint32_t)(w & 0x3FFFFFFFull); }
+
+// A neighbour at or above level k joins the list of vertex v at level k (a
+// new edge, or a neighbour that has just risen to k): v's record counts it
+// above, or appends it.  Runs between searches, when nobody reads records.
+__device__ __forceinline__ void rec_link(const MaintainParams& P, uint32_t e0, int v, int k, int other,
+                                         bool other_above) {
+    const unsigned long long w = vload64(&P.rec[v]);
+    if (rec_stamp(w) < e0) return;
+    int32_t* r = P.arena + 4 * (w >> 30);
+    const int room = vload32(&r[1]);
+    if (vload32(&r[3]) != k) return;
+    if (other_above) {
+        atomicAdd(&r[2], 1);
+        return;
+    }
+    const int at = atomicAdd(&r[0], 1);
+    if (at < room) r[4 + at] = other;
 }
+
+// Room for the ids of a record of a vertex with superior degree sd and a
+// list of len slots: its core-k neighbours number at most sd, and the rest is
+// for those that join.
+__device__ __forceinline__ int rec_room(int sd, int len) { return min(sd, len) + (sd >> 3) + 16; }
 
 // What a warp carries through a search besides its buffer.
 struct Walker {
     int nk;        // kept tasks
     int klim;      // most it may keep: 1 while warps wait for tasks, 32 while the queue is long
-    int nrec;      // records made but not published: lane i < nrec holds one
-    int rec_v;
-    unsigned long long rec_q;
-    unsigned long long slab, slab_end;   // arena quads it holds
+    bool more;     // iterations follow: records take the whole level, not the candidates alone
+    int nrec;      // records made but not published
 };
+
+// Arena room for n quads behind what the warp holds: the first quad, or
+// NO_QUAD.  A warp takes room in slabs, so few records touch the shared
+// counter; the caller moves B.slab past what it uses.  Warp-uniform.
+constexpr unsigned long long NO_QUAD = ~0ull;
+__device__ __forceinline__ unsigned long long arena_reserve(Ctl* C, const MaintainParams& P, WarpBuf& B, unsigned n) {
+    unsigned long long at = B.slab;
+    if (B.slab_end - at >= n) return at;
+    const unsigned long long q = n > P.slab_quads ? n : P.slab_quads;
+    if (lane_id() == 0) at = atomicAdd(&C->rec_top, q);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (at + q > P.arena_quads) return NO_QUAD;
+    if (lane_id() == 0) {
+        B.slab = at;
+        B.slab_end = at + q;
+    }
+    __syncwarp();
+    return at;
+}
 
 // ---------------------------------------------------------------- pushes
 // Appends the vertices of the lanes' bit masks (bit j: id[j]) to the logs
-// and the task queue: `fm` enter the frontier (insert), `em` are evicted.
-// One atomic per counter for the warp, issued by three lanes at once.  The
+// and the task queue: `fm` enter the frontier (insert), `em` are evicted (an
+// insertion needs no log of its evictions).  One atomic per counter for the
+// warp, issued by several lanes at once.  The
 // first few stay with the warp (W.klim): it runs them next, which saves the
 // hand-off through the queue.  A kept task is not counted in the queue's
 // tail and not reported done; the task that produced it is reported only
 // when the warp has run out of kept tasks, so quiescence still waits for it.
 // Evictions are kept first: they prune the search.  Warp-collective.
-template <int J>
+template <bool DEL, int J>
 __device__ __forceinline__ void push_new(Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W, unsigned fm,
                                          unsigned em, const int (&id)[J]) {
     if (!__any_sync(0xffffffffu, (fm | em) != 0)) return;
@@ -128,7 +201,8 @@ __device__ __forceinline__ void push_new(Ctl* C, const MaintainParams& P, WarpBu
     unsigned long long base = 0;
     if (lane < 3) {
         unsigned long long* p = lane == 0 ? &C->tail[0] : lane == 1 ? &C->tail[1] : &C->task_tail;
-        const unsigned long long n = lane == 0 ? (unsigned long long)nf : lane == 1 ? (unsigned long long)ne : nq;
+        const unsigned long long n = lane == 0 ? (unsigned long long)nf
+                                     : lane == 1 ? (unsigned long long)(DEL ? ne : 0) : nq;
         if (n) base = atomicAdd(p, n);
     }
     const unsigned long long fb = __shfl_sync(0xffffffffu, base, 0);
@@ -142,8 +216,9 @@ __device__ __forceinline__ void push_new(Ctl* C, const MaintainParams& P, WarpBu
         const bool f = (fm >> j) & 1u, x = (em >> j) & 1u;
         if (!f && !x) continue;
         const int rank = x ? er : ne + fr;
-        if (x) P.EQ[(eb + er++) & P.qmask] = id[j];
-        else P.VQ[(fb + fr++) & P.qmask] = id[j];
+        if (!x) P.VQ[(fb + fr++) & P.qmask] = id[j];
+        else if (DEL) P.EQ[(eb + er++) & P.qmask] = id[j];
+        else er++;
         const unsigned long long task = mk_task(x ? T_EVICT : T_FRONT, (unsigned long long)(uint32_t)id[j]);
         if (rank < kq) B.kept[W.nk + rank] = task;
         else if (room) vstore64(&P.TQ[(tb + (unsigned)(rank - kq)) & P.tqmask], task);
@@ -153,15 +228,22 @@ __device__ __forceinline__ void push_new(Ctl* C, const MaintainParams& P, WarpBu
 }
 
 // ---------------------------------------------------------------- scan of one list
-// Slots [s, min(s + 128 U, len)) of a list of a vertex at level k: adds
-// this lane's share of CSD to `part` (insert: the neighbours above k and the
-// candidates, Definition 8) and, if `store`, appends the candidates to the
-// buffer behind the nc it holds.  Returns the new count.  Lists start
-// 16-byte aligned and their capacity is a multiple of 4; they are read
-// evict-first so that L2 keeps the keys.  Warp-collective.
-template <bool DEL, int U = 4>
-__device__ __forceinline__ int scan_window(const DevGraph& g, const int32_t* list, int s, int len, int k, bool store,
-                                           WarpBuf& B, int nc, int& part) {
+// Slots [s, min(s + 128 U, len)) of a list (from_rec: of a record's ids).
+// The candidates go to the front of the buffer; returns their number.
+//   S_INSERT: the core-k neighbours with SD > k; `part` gains this lane's
+//             share of CSD (Definition 8: those and the neighbours above k),
+//             and with `others` the remaining core-k neighbours go to the end
+//             of the buffer, the last one first (their number: ne);
+//   S_DELETE: the core-k neighbours;
+//   S_ROSE, S_DROPPED: the neighbours of core k, whose SD counts a vertex
+//             differently now that it has risen to k or dropped to k - 1;
+//             `part` gains the share of that vertex's own SD.
+// Lists start 16-byte aligned and their capacity is a multiple of 4; they
+// are read evict-first so that L2 keeps the keys.  Warp-collective.
+enum { S_INSERT = 0, S_DELETE = 1, S_ROSE = 2, S_DROPPED = 3 };
+template <int KIND, int U = 4>
+__device__ __forceinline__ int scan_window(const DevGraph& g, const int32_t* list, bool from_rec, int s, int len,
+                                           int k, bool others, WarpBuf& B, int& part, int& ne) {
     const int lane = lane_id();
     int id[4 * U];
 #pragma unroll
@@ -169,7 +251,13 @@ __device__ __forceinline__ int scan_window(const DevGraph& g, const int32_t* lis
         const int t = s + u * 128 + lane * 4;
         int4 a = make_int4(HOLE, HOLE, HOLE, HOLE);
         if (t < len) a = __ldcs(reinterpret_cast<const int4*>(list + t));
-        id[4 * u] = a.x;
+        if (KIND == S_INSERT && from_rec) {
+            a.x &= ~REC_CAND;
+            a.y &= ~REC_CAND;
+            a.z &= ~REC_CAND;
+            a.w &= ~REC_CAND;
+        }
+        id[4 * u] = t < len ? a.x : HOLE;
         id[4 * u + 1] = t + 1 < len ? a.y : HOLE;
         id[4 * u + 2] = t + 2 < len ? a.z : HOLE;
         id[4 * u + 3] = t + 3 < len ? a.w : HOLE;
@@ -177,31 +265,38 @@ __device__ __forceinline__ int scan_window(const DevGraph& g, const int32_t* lis
     uint32_t key[4 * U];
 #pragma unroll
     for (int i = 0; i < 4 * U; i++) key[i] = id[i] >= 0 ? g.kc[id[i]] : KEY_DEAD;
-    unsigned mask = 0;
+    unsigned mask = 0, eq = 0;
 #pragma unroll
     for (int i = 0; i < 4 * U; i++) {
-        if (DEL) {
-            mask |= key_core(key[i]) == k ? 1u << i : 0u;
-        } else {   // key order is (core, bit): above k or a candidate <=> key >= 2k + 1
+        if (KIND == S_INSERT) {   // key order is (core, bit): above k or a candidate <=> key >= 2k + 1
             part += (int)key[i] >= 2 * k + 1;
             mask |= key[i] == (uint32_t)(2 * k + 1) ? 1u << i : 0u;
+            eq |= key[i] == (uint32_t)(2 * k) ? 1u << i : 0u;
+        } else {
+            if (KIND != S_DELETE) part += key_core(key[i]) >= (KIND == S_ROSE ? k : k - 1);
+            mask |= key_core(key[i]) == k ? 1u << i : 0u;
         }
     }
-    if (!store || !__any_sync(0xffffffffu, mask != 0)) return nc;
-    const int cnt = __popc(mask);
+    if (KIND != S_INSERT || !others) eq = 0;
+    ne = 0;
+    if (!__any_sync(0xffffffffu, (mask | eq) != 0)) return 0;
+    const int cnt = __popc(mask) | (__popc(eq) << 16);   // at most 512 of both together
     int incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += t;
     }
-    int at = nc + incl - cnt;
+    const int tot = __shfl_sync(0xffffffffu, incl, 31);
+    int at = (incl - cnt) & 0xFFFF, end = kWindow - 1 - ((incl - cnt) >> 16);
 #pragma unroll
-    for (int i = 0; i < 4 * U; i++)
+    for (int i = 0; i < 4 * U; i++) {
         if ((mask >> i) & 1u) B.id[at++] = id[i];
-    nc += __shfl_sync(0xffffffffu, incl, 31);
+        if (KIND == S_INSERT && ((eq >> i) & 1u)) B.id[end--] = id[i];
+    }
+    ne = tot >> 16;
     __syncwarp();
-    return nc;
+    return tot & 0xFFFF;
 }
 
 // ---------------------------------------------------------------- candidates
@@ -268,33 +363,44 @@ __device__ __forceinline__ void act_insert(const DevGraph& g, Ctl* C, const Main
             if (v) fm |= (wz(r[j]) & kVisited) == 0 ? 1u << j : 0u;
             else em |= (wz(r[j]) & kProcessed) && ww(r[j]) == kk[j] + 1 ? 1u << j : 0u;
         }
-        push_new<J>(C, P, B, W, fm, em, id);
+        push_new<false, J>(C, P, B, W, fm, em, id);
     }
 }
 
-// Recorded candidates [i0, i1) of an evicted vertex at level k.  Its own
-// expansion visited every one of them in this iteration (the record is
-// published after that), so their words carry the iteration's stamp and a
-// plain add does.  Warp-collective.
+// The recorded ids [i0, i1) of an evicted vertex at level k.  Its expansion
+// in this iteration visited the candidates among them, so their words carry
+// the iteration's stamp and a plain add does.  all: the record is of an
+// earlier iteration and its marks are out of date (ids have risen above k,
+// SDs have grown), so the keys tell who is a candidate now.  Warp-collective.
 __device__ __forceinline__ void act_recorded(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                             const int32_t* list, int i0, int i1, int k) {
+                                             const int32_t* list, int i0, int i1, int k, bool all) {
     const int lane = lane_id();
     for (int b0 = i0; b0 < i1; b0 += 128) {
         int id[4];
-        unsigned long long r[4];
+        unsigned go = 0, em = 0;
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             const int i = b0 + j * 32 + lane;
-            id[j] = i < i1 ? __ldcg(list + i) : -1;
+            const int x = i < i1 ? __ldcg(list + i) : 0;
+            id[j] = x & ~REC_CAND;
+            go |= i < i1 && (all || x < 0) ? 1u << j : 0u;
         }
+        if (all) {
+            uint32_t key[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) key[j] = (go >> j) & 1u ? g.kc[id[j]] : KEY_DEAD;
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (key[j] != (uint32_t)(2 * k + 1)) go &= ~(1u << j);
+        }
+        unsigned long long r[4];
 #pragma unroll
         for (int j = 0; j < 4; j++)
-            r[j] = id[j] >= 0 ? atomicAdd(iter_word(g, id[j]), 0xFFFFFFFF00000000ull) : 0ull;
-        unsigned em = 0;
+            r[j] = (go >> j) & 1u ? atomicAdd(iter_word(g, id[j]), 0xFFFFFFFF00000000ull) : 0ull;
 #pragma unroll
         for (int j = 0; j < 4; j++)
-            em |= id[j] >= 0 && (wz(r[j]) & kProcessed) && ww(r[j]) == k + 1 ? 1u << j : 0u;
-        push_new<4>(C, P, B, W, 0u, em, id);
+            em |= ((go >> j) & 1u) && (wz(r[j]) & kProcessed) && ww(r[j]) == k + 1 ? 1u << j : 0u;
+        push_new<false, 4>(C, P, B, W, 0u, em, id);
     }
 }
 
@@ -349,16 +455,17 @@ __device__ __forceinline__ void act_delete(const DevGraph& g, Ctl* C, const Main
                 em |= 1u << j;
             }
         }
-        push_new<J>(C, P, B, W, 0u, em, id);
+        push_new<true, J>(C, P, B, W, 0u, em, id);
     }
 }
 
 // ---------------------------------------------------------------- hub items
 // Creates a hub item and its chunk tasks (warp-collective); false if the
-// item ring is full (the caller then scans the list itself).  sd > 0: the
-// item also reserves arena room for sd recorded candidates.
+// item ring is full (the caller then walks the list itself).  acc0: what its
+// sum starts from; room > 0: the item also reserves arena room for a record
+// of that many ids.
 __device__ __forceinline__ bool make_hub(Ctl* C, const MaintainParams& P, int v, int kind, int k, long long off,
-                                         int len, int sd) {
+                                         int len, int acc0, int room) {
     const int lane = lane_id();
     const int nch = (len + kChunk - 1) / kChunk;
     unsigned long long idx = 0, tb = 0;
@@ -368,10 +475,10 @@ __device__ __forceinline__ bool make_hub(Ctl* C, const MaintainParams& P, int v,
             idx = atomicAdd(&C->hub_created, 1ull);
             unsigned long long rb = 0;
             int rcap = 0;
-            if (sd > 0) {
-                const unsigned long long q = 1ull + (unsigned long long)((sd + 3) >> 2);
+            if (room > 0) {
+                const unsigned long long q = 1ull + (unsigned long long)((room + 3) >> 2);
                 rb = atomicAdd(&C->rec_top, q);
-                if (rb + q <= P.arena_quads) rcap = sd;
+                if (rb + q <= P.arena_quads) rcap = room;
             }
             HubItem* it = &P.HQ[idx & (kHubRing - 1)];
             it->off = off;
@@ -380,9 +487,10 @@ __device__ __forceinline__ bool make_hub(Ctl* C, const MaintainParams& P, int v,
             it->k = k;
             it->len = len;
             it->nch = nch;
-            it->acc = 0;
+            it->acc = acc0;
             it->done = 0u;
             it->rcur = 0;
+            it->ncand = 0;
             it->rquad = rb;
             it->rcap = rcap;
             __threadfence();   // the item before its tasks
@@ -404,12 +512,127 @@ __device__ __forceinline__ bool make_hub(Ctl* C, const MaintainParams& P, int v,
 // One vertex pushed by the warp (an evicted hub).
 __device__ __forceinline__ void push_evicted(Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W, int v) {
     const int id[1] = {v};
-    push_new<1>(C, P, B, W, 0u, lane_id() == 0 ? 1u : 0u, id);
+    push_new<false, 1>(C, P, B, W, 0u, lane_id() == 0 ? 1u : 0u, id);
 }
 
-// One chunk task (warp-collective).
+// Adds a frontier vertex's CSD to its support and sets its processed flag;
+// returns the old word.  Whoever made it a frontier vertex stamped its word
+// with this iteration, so a plain add does.
+__device__ __forceinline__ unsigned long long add_csd(const DevGraph& g, int v, int csd) {
+    return atomicAdd(iter_word(g, v), ((unsigned long long)(uint32_t)csd << 32) + (unsigned long long)kProcessed);
+}
+
+// ---------------------------------------------------------------- one list walked by a warp
+// Slots [s0, s1) of a list (from_rec: of a record) of a vertex at level k,
+// window by window: scan, copy what belongs into a record, act on the
+// candidates.  The one place for all insertion walks of single lists (whole
+// lists, records, chunks of hubs), so that its instructions stay cached.
+enum { A_EVICT = 0, A_VISIT = 1, A_COUNT = 2 };
+struct Walk {
+    const int32_t* list;
+    int s0, s1, k;
+    bool from_rec;
+    int act;
+    int32_t* out;     // ids of the record being made (NULL: none)
+    int room;         // ... and room for them; past it `nrec` counts on
+    int* shared;      // ... a hub's: the ids so far, shared by its chunks
+    // results
+    int part, ncand, nrec;
+};
+__device__ __forceinline__ void walk_insert(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                            Walk& L, uint32_t e) {
+    const int lane = lane_id();
+    L.part = L.ncand = L.nrec = 0;
+    for (int s = L.s0; s < L.s1; s += kWindow) {
+        int ne = 0;
+        const int nc = scan_window<S_INSERT>(g, L.list, L.from_rec, s, L.s1, L.k, L.out && W.more, B, L.part, ne);
+        L.ncand += nc;
+        if (L.out && nc + ne > 0) {
+            int at = L.nrec;
+            L.nrec += nc + ne;
+            if (L.shared) {
+                if (lane == 0) at = atomicAdd(L.shared, nc + ne);
+                at = __shfl_sync(0xffffffffu, at, 0);
+            }
+            if (at + nc + ne <= L.room) {
+                for (int i = lane; i < nc; i += 32) L.out[at + i] = B.id[i] | REC_CAND;
+                for (int i = lane; i < ne; i += 32) L.out[at + nc + i] = B.id[kWindow - 1 - i];
+            }
+        }
+        if (L.act != A_COUNT && nc > 0)
+            act_insert<false>(g, C, P, B, W, nc, L.k, e, [&] { return (unsigned)L.act; });
+        __syncwarp();   // the buffer is free again
+    }
+}
+
+// Makes a record of the walk's ids at arena quad q (header; the ids are
+// there), room for `room` of them.  One lane calls it.
+__device__ __forceinline__ void rec_header(const MaintainParams& P, const Walker& W, unsigned long long q, int n,
+                                           int room, int above, int k) {
+    *reinterpret_cast<int4*>(P.arena + 4 * q) = make_int4(n, room, above, W.more ? k : -1);
+}
+
+// Publishes the records a warp has made (at most 32), with one
+// fence for all of them.  A vertex that is evicted before its record is out
+// has its list walked again.
+__device__ __forceinline__ void publish_records(const MaintainParams& P, WarpBuf& B, Walker& W, uint32_t e) {
+    if (W.nrec == 0) return;
+    __syncwarp();
+    __threadfence();
+    if (lane_id() < W.nrec) vstore64(&P.rec[B.rec_v[lane_id()]], rec_word(B.rec_q[lane_id()], e));
+    W.nrec = 0;
+}
+
+// A frontier vertex with more than kShort slots (Algorithm 3): support +=
+// CSD; above k it visits its candidates, else it is evicted.  Nearly all of
+// them survive, so the candidates are visited as they are found
+// (expand_early); one that fails after all, or the paper's order, walks the
+// list again.  A list is recorded; from_rec: `list` is the vertex's record,
+// `above` the neighbours it counts above k.
+__device__ __forceinline__ void long_front(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
+                                           int v, int k, const int32_t* list, int len, bool from_rec, int above,
+                                           int room, uint32_t e) {
+    const int lane = lane_id();
+    const bool early = expand_early(P);
+    unsigned long long q = NO_QUAD;
+    if (!from_rec) q = arena_reserve(C, P, B, 1u + (unsigned)((room + 3) >> 2));
+    Walk L{list, 0, len, k, from_rec, early ? A_VISIT : A_COUNT, q != NO_QUAD ? P.arena + 4 * q + 4 : nullptr, room,
+           nullptr, 0, 0, 0};
+    for (;;) {
+        walk_insert(g, C, P, B, W, L, e);
+        if (L.act == A_EVICT || (L.act == A_VISIT && !early)) break;   // the second walk
+        const int csd = warp_sum(L.part) + above;
+        unsigned up = 0;
+        if (lane == 0) {
+            up = ww(add_csd(g, v, csd)) + csd > k ? 1u : 0u;
+            note(B, N_VIS, 1);
+            note(B, N_VISL, len);
+            if (!up) note(B, N_EV, 1);
+        }
+        up = __shfl_sync(0xffffffffu, up, 0);
+        if (L.out && L.nrec <= room) {
+            const int keep = min(room, W.more ? L.nrec + (L.nrec >> 2) + 16 : L.nrec);
+            if (lane == 0) {
+                rec_header(P, W, q, L.nrec, keep, csd - L.ncand, k);
+                B.slab = q + 1 + (unsigned)((keep + 3) >> 2);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                B.rec_v[W.nrec] = v;
+                B.rec_q[W.nrec] = q;
+            }
+            W.nrec++;
+        }
+        if (early && up) break;
+        L.out = nullptr;
+        L.act = up ? A_VISIT : A_EVICT;
+    }
+}
+
+// One chunk task of a hub (warp-collective).
+template <bool DEL>
 __device__ __forceinline__ void run_chunk(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                          uint32_t e, LocalStats& ls, unsigned long long payload) {
+                                          uint32_t e, unsigned long long payload) {
     const int lane = lane_id();
     HubItem* it = &P.HQ[payload >> kTaskChunkBits];
     const int ci = (int)(payload & ((1ull << kTaskChunkBits) - 1));
@@ -419,224 +642,101 @@ __device__ __forceinline__ void run_chunk(const DevGraph& g, Ctl* C, const Maint
     const long long off = (long long)vload64((const unsigned long long*)&it->off);
     const unsigned long long rquad = vload64(&it->rquad);
     const int s0 = ci * kChunk, s1 = min(s0 + kChunk, len);
-    if (kind == HUB_FRONT || kind == HUB_FRONT_SPEC) {
-        const bool spec = kind == HUB_FRONT_SPEC;
-        int part = 0;
-        const int nc = scan_window<false>(g, g.adj + off, s0, s1, k, spec, B, 0, part);
-        part = warp_sum(part);
-        if (spec && nc > 0) {
-            int at = 0;
-            if (lane == 0 && rcap > 0) at = atomicAdd(&it->rcur, nc);
-            at = __shfl_sync(0xffffffffu, at, 0);
-            if (rcap > 0 && at + nc <= rcap) {
-                int32_t* out = P.arena + 4 * rquad + 4 + at;
-                for (int i = lane; i < nc; i += 32) out[i] = B.id[i];
-            }
-            act_insert<false>(g, C, P, B, W, nc, k, e, [] { return 1u; });
-        }
-        __syncwarp();
-        int decide = 0;   // 1 expand, 2 evict
-        if (lane == 0) {
+    const bool front = kind == HUB_FRONT || kind == HUB_FRONT_SPEC || kind == HUB_FRONT_REC;
+    int part = 0, ncand = 0;
+    if constexpr (DEL) {
+        int ne = 0;
+        const int nc = scan_window<S_DELETE>(g, g.adj + off, false, s0, s1, k, false, B, part, ne);
+        act_delete<false>(g, C, P, B, W, nc, k, e);
+    } else if (kind == HUB_EVICT_REC) {
+        act_recorded(g, C, P, B, W, P.arena + off, s0, s1, k, vload32i(&it->acc) != 0);
+    } else {
+        Walk L{(kind == HUB_FRONT_REC ? P.arena : g.adj) + off, s0, s1, k, kind == HUB_FRONT_REC,
+               kind == HUB_FRONT ? A_COUNT : kind == HUB_EVICT_INS ? A_EVICT : A_VISIT,
+               rcap > 0 ? P.arena + 4 * rquad + 4 : nullptr, rcap, &it->rcur, 0, 0, 0};
+        walk_insert(g, C, P, B, W, L, e);
+        ncand = L.ncand;
+        part = warp_sum(L.part);
+    }
+    __syncwarp();
+    int decide = 0;   // 1 expand, 2 evict
+    if (lane == 0) {
+        if (front) {
             atomicAdd(&it->acc, part);
-            __threadfence();
-            if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
+            if (ncand) atomicAdd(&it->ncand, ncand);
+        }
+        __threadfence();
+        if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
+            if (front) {
                 __threadfence();
                 const int acc = atomicAdd(&it->acc, 0);
                 const int rcur = atomicAdd(&it->rcur, 0);
                 if (rcap > 0 && rcur <= rcap) {   // the record before the flag that lets others evict v
-                    P.arena[4 * rquad] = rcur;
+                    rec_header(P, W, rquad, rcur, rcap, acc - atomicAdd(&it->ncand, 0), k);
                     __threadfence();
                     vstore64(&P.rec[v], rec_word(rquad, e));
                 }
-                uint32_t of;
-                int32_t oc;
-                add_word(g, C, v, e, acc, kProcessed, of, oc);
-                ls.vis++;
-                ls.visl += len;
-                decide = oc + acc > k ? 1 : 2;
-                atomicAdd(&C->hub_finished, 1ull);
-            }
-        }
-        decide = __shfl_sync(0xffffffffu, decide, 0);
-        if (decide == 1 && !spec && !make_hub(C, P, v, HUB_EXPAND, k, off, len, 0)) {
-            for (int s = 0; s < len; s += kWindow) {
-                const int m = scan_window<false>(g, g.adj + off, s, len, k, true, B, 0, part);
-                act_insert<false>(g, C, P, B, W, m, k, e, [] { return 1u; });
-            }
-        }
-        if (decide == 2) push_evicted(C, P, B, W, v);
-        return;
-    }
-    int unused = 0;
-    if (kind == HUB_EVICT_REC) {
-        act_recorded(g, C, P, B, W, P.arena + off, s0, s1, k);
-    } else if (kind == HUB_EVICT_DEL) {
-        const int nc = scan_window<true>(g, g.adj + off, s0, s1, k, true, B, 0, unused);
-        act_delete<false>(g, C, P, B, W, nc, k, e);
-    } else {   // HUB_EXPAND visits, HUB_EVICT_INS evicts
-        const int nc = scan_window<false>(g, g.adj + off, s0, s1, k, true, B, 0, unused);
-        act_insert<false>(g, C, P, B, W, nc, k, e, [&] { return kind == HUB_EXPAND ? 1u : 0u; });
-    }
-    __syncwarp();
-    if (lane == 0) {
-        __threadfence();
-        if (atomicAdd(&it->done, 1u) == (uint32_t)(nch - 1)) {
-            if (kind == HUB_EVICT_DEL) {
-                g.hc[v].x = k - 1;
-                g.kc[v] = key_of(k - 1, 0);   // the SD fix-up of the next claim phase sets its bit
-            }
-            if (kind != HUB_EXPAND) {
-                ls.ev++;
-                ls.evl += len;
+                decide = ww(add_csd(g, v, acc)) + acc > k ? 1 : 2;
+                note(B, N_VIS, 1);
+                note(B, N_VISL, len);
+            } else if (kind != HUB_EXPAND) {
+                if (DEL) {
+                    g.hc[v].x = k - 1;
+                    g.kc[v] = key_of(k - 1, 0);   // the SD fix-up of the next claim phase sets its bit
+                }
+                note(B, N_EV, 1);
+                note(B, N_EVL, len);
             }
             atomicAdd(&C->hub_finished, 1ull);
         }
     }
-}
-
-// ---------------------------------------------------------------- single lists
-// Adds a frontier vertex's CSD to its support and sets its processed flag;
-// returns the old word.  Whoever made it a frontier vertex stamped its word
-// with this iteration, so a plain add does.
-__device__ __forceinline__ unsigned long long add_csd(const DevGraph& g, int v, int csd) {
-    return atomicAdd(iter_word(g, v), ((unsigned long long)(uint32_t)csd << 32) + (unsigned long long)kProcessed);
-}
-
-// Arena room for n candidates and their count: the first quad, or NO_QUAD.
-// A warp takes room in slabs, so few records touch the shared counter; what
-// is left of a slab too small for a record is dropped.  Warp-uniform result.
-constexpr unsigned long long NO_QUAD = ~0ull;
-__device__ __forceinline__ unsigned long long arena_take(Ctl* C, const MaintainParams& P, Walker& W, int n) {
-    const unsigned need = 1u + (unsigned)((n + 3) >> 2);
-    if (W.slab_end - W.slab < need) {
-        const unsigned long long q = need > P.slab_quads ? need : P.slab_quads;
-        unsigned long long at = 0;
-        if (lane_id() == 0) at = atomicAdd(&C->rec_top, q);
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (at + q > P.arena_quads) return NO_QUAD;
-        W.slab = at;
-        W.slab_end = at + q;
+    if constexpr (!DEL) {
+        decide = __shfl_sync(0xffffffffu, decide, 0);
+        if (decide == 1 && kind == HUB_FRONT && !make_hub(C, P, v, HUB_EXPAND, k, off, len, 0, 0)) {
+            Walk L{g.adj + off, 0, len, k, false, A_VISIT, nullptr, 0, nullptr, 0, 0, 0};
+            walk_insert(g, C, P, B, W, L, e);
+        }
+        if (decide == 2) push_evicted(C, P, B, W, v);
     }
-    const unsigned long long q = W.slab;
-    W.slab += need;
-    return q;
 }
 
-// A frontier vertex with more than kShort slots (Algorithm 3): support +=
-// CSD; above k it visits its candidates and leaves a record of them (W.rec_*:
-// published by publish_records), else it is evicted.  Nearly all of them
-// survive this step, so the candidates are visited while the support atomic
-// is under way (expand_early); one that fails after all then evicts from the
-// same buffer.  A list whose candidates do not fit the buffer (only without
-// hub items, or with a larger hub_len) is scanned again to act.
-__device__ __forceinline__ void long_front(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                           int v, int k, const int32_t* list, int len, uint32_t e, LocalStats& ls) {
-    const int lane = lane_id();
-    int nc = 0, part = 0;
-    bool spilled = false;
+// A vertex with more than kShort slots evicted by a deletion (Algorithm 7):
+// it drops to k - 1.
+__device__ __forceinline__ void long_evict_delete(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B,
+                                                  Walker& W, int v, int k, const int32_t* list, int len,
+                                                  uint32_t e) {
+    int part = 0, ne = 0;
     for (int s = 0; s < len; s += kWindow) {
-        spilled = spilled || nc + kWindow > kCand;
-        nc = scan_window<false>(g, list, s, len, k, !spilled, B, nc, part);
-    }
-    const int csd = warp_sum(part);
-    unsigned long long old = 0;
-    if (lane == 0) {
-        old = add_csd(g, v, csd);
-        ls.vis++;
-        ls.visl += len;
-    }
-    auto above = [&] { return __shfl_sync(0xffffffffu, ww(old) + csd > k ? 1u : 0u, 0); };
-    if (spilled) {
-        const unsigned up = above();
-        for (int s = 0; s < len; s += kWindow) {
-            const int m = scan_window<false>(g, list, s, len, k, true, B, 0, part);
-            act_insert<false>(g, C, P, B, W, m, k, e, [&] { return up; });
-        }
-        if (!up && lane == 0) ls.ev++;
-        return;
-    }
-    const bool early = expand_early(P);
-    if (nc > 0) {
-        const unsigned long long q = arena_take(C, P, W, nc);
-        if (q != NO_QUAD) {
-            int32_t* out = P.arena + 4 * q;
-            if (lane == 0) out[0] = nc;
-            for (int i = lane; i < nc; i += 32) out[4 + i] = B.id[i];
-        }
-        unsigned up = 1u;
-        act_insert<false>(g, C, P, B, W, nc, k, e, [&] {
-            if (!early) up = above();
-            return up;
-        });
-        if (early) {
-            up = above();
-            if (!up) act_insert<false>(g, C, P, B, W, nc, k, e, [] { return 0u; });
-        }
-        if (!up && lane == 0) ls.ev++;
-        // the record is complete, and every candidate carries the iteration's stamp
-        if (up && q != NO_QUAD) {
-            if (lane == W.nrec) {
-                W.rec_v = v;
-                W.rec_q = q;
-            }
-            W.nrec++;
-        }
-        return;
-    }
-    if (!above() && lane == 0) ls.ev++;
-}
-
-// Publishes the records a warp has made (at most one per lane), with one
-// fence for all of them.  A vertex that is evicted before its record is out
-// has its list scanned again.
-__device__ __forceinline__ void publish_records(const MaintainParams& P, Walker& W, uint32_t e) {
-    if (W.nrec == 0) return;
-    __syncwarp();
-    __threadfence();
-    if (lane_id() < W.nrec) vstore64(&P.rec[W.rec_v], rec_word(W.rec_q, e));
-    W.nrec = 0;
-}
-
-// An evicted vertex with more than kShort slots (insert: Algorithm 4; delete:
-// Algorithm 7, the vertex drops to k - 1).
-template <bool DEL>
-__device__ __forceinline__ void long_evict(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                           int v, int k, const int32_t* list, int len, uint32_t e, LocalStats& ls) {
-    int unused = 0;
-    for (int s = 0; s < len; s += kWindow) {
-        const int m = scan_window<DEL>(g, list, s, len, k, true, B, 0, unused);
-        if (DEL) act_delete<false>(g, C, P, B, W, m, k, e);
-        else act_insert<false>(g, C, P, B, W, m, k, e, [] { return 0u; });
+        const int nc = scan_window<S_DELETE>(g, list, false, s, len, k, false, B, part, ne);
+        act_delete<false>(g, C, P, B, W, nc, k, e);
+        __syncwarp();
     }
     if (lane_id() == 0) {
-        if (DEL) {
-            g.hc[v].x = k - 1;
-            g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
-        }
-        ls.ev++;
-        ls.evl += len;
+        g.hc[v].x = k - 1;
+        g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
+        note(B, N_EV, 1);
+        note(B, N_EVL, len);
     }
 }
 
-// A task with at most kShort slots that is alone in its batch: one scan
+// A task with at most 128 slots that is alone in its batch: one scan
 // step, and one candidate per lane where they fit (the walk of many short
 // lists takes about three times the instructions, which is what a lone task's
 // latency consists of once its words are in L2).
 template <bool DEL>
 __device__ __forceinline__ void lone_short(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                           int v, int k, const int32_t* list, int len, bool front, uint32_t e,
-                                           LocalStats& ls) {
+                                           int v, int k, const int32_t* list, int len, bool front, uint32_t e) {
     const int lane = lane_id();
-    int part = 0;
-    const int nc = scan_window<DEL, 1>(g, list, 0, len, k, true, B, 0, part);
+    int part = 0, ne = 0;
+    const int nc = scan_window<DEL ? S_DELETE : S_INSERT, 1>(g, list, false, 0, len, k, false, B, part, ne);
     if constexpr (DEL) {
         if (nc <= 32) act_delete<false, 1>(g, C, P, B, W, nc, k, e);
         else act_delete<false, 4>(g, C, P, B, W, nc, k, e);
         if (lane == 0) {
             g.hc[v].x = k - 1;
             g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
-            ls.ev++;
-            ls.evl += len;
+            note(B, N_EV, 1);
+            note(B, N_EVL, len);
         }
     } else {
         unsigned long long old = 0;
@@ -645,17 +745,17 @@ __device__ __forceinline__ void lone_short(const DevGraph& g, Ctl* C, const Main
             csd = warp_sum(part);
             if (lane == 0) {
                 old = add_csd(g, v, csd);
-                ls.vis++;
-                ls.visl += len;
+                note(B, N_VIS, 1);
+                note(B, N_VISL, len);
             }
         } else if (lane == 0) {
-            ls.ev++;
-            ls.evl += len;
+            note(B, N_EV, 1);
+            note(B, N_EVL, len);
         }
         auto decide = [&] {
             if (!front) return 0u;
             const unsigned up = __shfl_sync(0xffffffffu, ww(old) + csd > k ? 1u : 0u, 0);
-            if (!up && lane == 0) ls.ev++;
+            if (!up && lane == 0) note(B, N_EV, 1);
             return up;
         };
         if (nc <= 32) act_insert<false, 1>(g, C, P, B, W, nc, k, e, decide);
@@ -667,13 +767,13 @@ __device__ __forceinline__ void lone_short(const DevGraph& g, Ctl* C, const Main
 // Runs the tasks of the lanes with t != TASK_EMPTY (warp-collective).
 template <bool DEL>
 __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                          uint32_t e, LocalStats& ls, unsigned long long t) {
+                                          uint32_t e, uint32_t e0, unsigned long long t) {
     const int lane = lane_id();
     const bool have = t != TASK_EMPTY;
     const int type = have ? (int)(t >> 62) : -1;
     for (unsigned m = __ballot_sync(0xffffffffu, type == T_CHUNK); m; m &= m - 1) {
         const unsigned long long payload = __shfl_sync(0xffffffffu, t, __ffs(m) - 1) & ((1ull << 62) - 1);
-        run_chunk(g, C, P, B, W, e, ls, payload);
+        run_chunk<DEL>(g, C, P, B, W, e, payload);
     }
     const bool vert = type == T_FRONT || type == T_EVICT;
     if (!__any_sync(0xffffffffu, vert)) return;
@@ -686,10 +786,16 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
         const int2 c = g.hc[v];
         off = g.off[v];
         len = g.end[v];
-        if (!DEL && !front) rec = ld_acquire64(&P.rec[v]);
+        if (!DEL) rec = ld_acquire64(&P.rec[v]);
         k = c.x;
         sd = c.y;
     }
+    int4 hdr = make_int4(0, 0, 0, -1);
+    if (!DEL && vert && len > kShort && rec_stamp(rec) >= e0)
+        hdr = __ldcg(reinterpret_cast<const int4*>(P.arena + 4 * (rec >> 30)));
+    // whose record will do: at its level k, or made in this very iteration
+    const bool now = rec_stamp(rec) == e;
+    const unsigned use = __ballot_sync(0xffffffffu, hdr.x <= hdr.y && hdr.y > 0 && (hdr.w == k || (now && !front)));
     // lists of more than kShort slots, one after another
     for (unsigned m = __ballot_sync(0xffffffffu, vert && len > kShort); m; m &= m - 1) {
         const int src = __ffs(m) - 1;
@@ -698,42 +804,50 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
         const long long xoff = __shfl_sync(0xffffffffu, off, src);
         const bool xfront = __shfl_sync(0xffffffffu, (int)front, src) != 0;
         const bool hub = P.hub_len > 0 && xlen >= P.hub_len;
-        if (DEL) {
-            if (!hub || !make_hub(C, P, xv, HUB_EVICT_DEL, xk, xoff, xlen, 0))
-                long_evict<true>(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e, ls);
-            continue;
-        }
-        if (xfront) {
-            const int xsd = __shfl_sync(0xffffffffu, sd, src);
-            const bool spec = expand_early(P);
-            if (!hub || !make_hub(C, P, xv, spec ? HUB_FRONT_SPEC : HUB_FRONT, xk, xoff, xlen, spec ? xsd : 0))
-                long_front(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e, ls);
-            continue;
-        }
-        unsigned long long q = 0;
-        if (rec_of(__shfl_sync(0xffffffffu, rec, src), e, q)) {
-            const int cnt = __ldcg(P.arena + 4 * q);
-            if (P.hub_len > 0 && cnt >= P.hub_len &&
-                make_hub(C, P, xv, HUB_EVICT_REC, xk, (long long)(4 * q + 4), cnt, 0))
-                continue;
-            act_recorded(g, C, P, B, W, P.arena + 4 * q + 4, 0, cnt, xk);
-            if (lane == 0) {
-                ls.ev++;
-                ls.evl += cnt;
+        if constexpr (DEL) {
+            if (!hub || !make_hub(C, P, xv, HUB_EVICT_DEL, xk, xoff, xlen, 0, 0))
+                long_evict_delete(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e);
+        } else {
+            const bool from_rec = ((use >> src) & 1u) != 0;
+            const long long ro = (long long)(4 * (__shfl_sync(0xffffffffu, rec, src) >> 30) + 4);
+            const int cnt = from_rec ? __shfl_sync(0xffffffffu, hdr.x, src) : xlen;
+            const bool big = from_rec ? P.hub_len > 0 && cnt >= P.hub_len : hub;
+            if (xfront) {
+                const int above = from_rec ? __shfl_sync(0xffffffffu, hdr.z, src) : 0;
+                const int room = rec_room(__shfl_sync(0xffffffffu, sd, src), xlen);
+                const bool spec = expand_early(P);
+                if (!big || !make_hub(C, P, xv, from_rec ? HUB_FRONT_REC : spec ? HUB_FRONT_SPEC : HUB_FRONT, xk,
+                                      from_rec ? ro : xoff, cnt, above, spec && !from_rec ? room : 0))
+                    long_front(g, C, P, B, W, xv, xk, from_rec ? P.arena + ro : g.adj + xoff, cnt, from_rec, above,
+                               room, e);
+            } else {
+                const int all = __shfl_sync(0xffffffffu, now ? 0 : 1, src);
+                if (!big || !make_hub(C, P, xv, from_rec ? HUB_EVICT_REC : HUB_EVICT_INS, xk, from_rec ? ro : xoff,
+                                      cnt, all, 0)) {
+                    if (from_rec) {
+                        act_recorded(g, C, P, B, W, P.arena + ro, 0, cnt, xk, all != 0);
+                    } else {
+                        Walk L{g.adj + xoff, 0, xlen, xk, false, A_EVICT, nullptr, 0, nullptr, 0, 0, 0};
+                        walk_insert(g, C, P, B, W, L, e);
+                    }
+                    if (lane == 0) {
+                        note(B, N_EV, 1);
+                        note(B, N_EVL, cnt);
+                    }
+                }
             }
-        } else if (!hub || !make_hub(C, P, xv, HUB_EVICT_INS, xk, xoff, xlen, 0)) {
-            long_evict<false>(g, C, P, B, W, xv, xk, g.adj + xoff, xlen, e, ls);
         }
     }
-    publish_records(P, W, e);
-    // the others together, up to 128 quads a window
+    publish_records(P, B, W, e);
+    // the others together, up to 128 quads (512 slots) a window
     unsigned rest = __ballot_sync(0xffffffffu, vert && len <= kShort);
     if (!rest) return;
-    if ((rest & (rest - 1)) == 0) {   // one: searches spend their thin phases here, so take the fewest steps
+    if ((rest & (rest - 1)) == 0 && __shfl_sync(0xffffffffu, len, __ffs(rest) - 1) <= 128) {
+        // one: searches spend their thin phases here, so take the fewest steps
         const int src = __ffs(rest) - 1;
         lone_short<DEL>(g, C, P, B, W, __shfl_sync(0xffffffffu, v, src), __shfl_sync(0xffffffffu, k, src),
                         g.adj + __shfl_sync(0xffffffffu, off, src), __shfl_sync(0xffffffffu, len, src),
-                        __shfl_sync(0xffffffffu, (int)front, src) != 0, e, ls);
+                        __shfl_sync(0xffffffffu, (int)front, src) != 0, e);
         return;
     }
     const int nq = vert && len <= kShort ? (len + 3) >> 2 : 0;
@@ -745,7 +859,7 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
     }
     int gbase = 0;
     while (rest) {
-        const bool in = ((rest >> lane) & 1u) && incl - gbase <= 128;   // at least one: a list has <= 32 quads
+        const bool in = ((rest >> lane) & 1u) && incl - gbase <= 128;   // at least one: a list has <= 64 quads
         const unsigned gm = __ballot_sync(0xffffffffu, in);
         const int gend = __shfl_sync(0xffffffffu, incl, 31 - __clz(gm));
         B.csd[lane] = 0;
@@ -812,8 +926,11 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
             if (in) {
                 g.hc[v].x = k - 1;
                 g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
-                ls.ev++;
-                ls.evl += len;
+            }
+            const uint32_t el = __reduce_add_sync(0xffffffffu, in ? (unsigned)len : 0u);
+            if (lane == 0) {
+                note(B, N_EV, (uint32_t)__popc(gm));
+                note(B, N_EVL, el);
             }
         } else {
             int csd = 0;
@@ -821,16 +938,20 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
             if (in && front) {
                 csd = B.csd[lane];
                 old = add_csd(g, v, csd);
-                ls.vis++;
-                ls.visl += len;
-            } else if (in) {
-                ls.ev++;
-                ls.evl += len;
+            }
+            const unsigned fronts = __ballot_sync(0xffffffffu, in && front);
+            const uint32_t fl = __reduce_add_sync(0xffffffffu, in && front ? (unsigned)len : 0u);
+            const uint32_t el = __reduce_add_sync(0xffffffffu, in && !front ? (unsigned)len : 0u);
+            if (lane == 0) {
+                note(B, N_VIS, (uint32_t)__popc(fronts));
+                note(B, N_VISL, fl);
+                note(B, N_EV, (uint32_t)__popc(gm & ~fronts));
+                note(B, N_EVL, el);
             }
             act_insert<true>(g, C, P, B, W, nc, k, e, [&] {
-                const bool up = in && front && ww(old) + csd > k;
-                if (in && front && !up) ls.ev++;
-                return __ballot_sync(0xffffffffu, up);
+                const unsigned up = __ballot_sync(0xffffffffu, in && front && ww(old) + csd > k);
+                if (lane == 0) note(B, N_EV, (uint32_t)__popc(fronts & ~up));
+                return up;
             });
         }
         __syncwarp();
@@ -839,8 +960,9 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
     }
 }
 
-// Search (iteration number) whose queue the block's poller found quiescent.
+// Search (iteration number) whose queue the block knows to be quiescent.
 __shared__ volatile uint32_t s_quiet;
+__shared__ unsigned long long s_search_t0;   // when the search began (its waits are bounded)
 
 // Drains the task queue (every warp of the grid).  Returns false on error.
 // A warp claims slots for its lanes with one atomic and polls them together;
@@ -855,22 +977,21 @@ __shared__ volatile uint32_t s_quiet;
 // reference, which put both in local memory.
 template <bool DEL>
 __device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const MaintainParams& P, uint32_t e,
-                                             LocalStats& ls) {
+                                             uint32_t e0, bool more) {
     const int lane = lane_id();
     WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
-    const unsigned long long t_start = gtimer();
-    const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
     const unsigned long long share = (unsigned long long)(P.claim_max > 1 ? P.claim_max : 1);
-    unsigned long long idx = 0, ndone = 0;
+    unsigned long long idx = 0;
+    unsigned ndone = 0;
     unsigned held = 0;   // lanes that hold a claimed slot
     int claim = 1;
     unsigned int nap = 32;
-    Walker W{0, 1, 0, 0, 0ull, 0ull, 0ull};
-    // one warp per block tests quiescence and tells the others through
-    // shared memory: a test reads two hot counters, and thousands of
-    // waiting warps reading them would slow the claims and pushes that
-    // share those counters' L2 slices
-    const bool poller = threadIdx.x < 32;
+    Walker W{0, 1, more, 0};
+    // One warp of the grid tests quiescence (a test reads two counters that
+    // every claim and push needs, so hundreds of testers slow those down);
+    // one warp per block watches the word it sets and tells the others
+    // through shared memory.
+    const bool watcher = threadIdx.x < 32, poller = watcher && blockIdx.x == 0;
     for (unsigned int spins = 0;; spins++) {
         unsigned long long t = TASK_EMPTY, h = 0, tl = 0;
         bool look = false;   // the backlog was read in this round
@@ -900,19 +1021,16 @@ __device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const Ma
                 if (lane == 0) {
                     if (ndone) {   // report before waiting
                         __threadfence();
-                        atomicAdd(&C->task_done, ndone);
+                        atomicAdd(&C->task_done, (unsigned long long)ndone);
                     }
                     if (poller) {
                         // quiescent: every task pushed has finished (done read first)
                         const unsigned long long d = ld_acquire64(&C->task_done);   // read before the tail
-                        if (d == vload64(&C->task_tail) || vload32(&C->error)) {
-                            s_quiet = e;
-                            quit = 1;
-                        }
-                    } else if (s_quiet == e) {
-                        quit = 1;
+                        if (d == vload64(&C->task_tail)) vstore64(&C->quiet, e);
                     }
-                    if (!quit && (spins & 3u) == 0 && gtimer() - t_start > P.limit_ns) {
+                    if (watcher && (vload64(&C->quiet) == e || vload32(&C->error))) s_quiet = e;
+                    if (s_quiet == e) quit = 1;
+                    if (!quit && (spins & 3u) == 0 && gtimer() - s_search_t0 > P.limit_ns) {
                         atomicCAS(&C->error, 0, E_BARRIER_TIMEOUT);
                         quit = 1;
                     }
@@ -928,7 +1046,7 @@ __device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const Ma
             nap = 32;
             if (t != TASK_EMPTY) vstore64(slot, TASK_EMPTY);   // free for the next search
             held &= ~got;
-            ndone += (unsigned long long)__popc(got);
+            ndone += (unsigned)__popc(got);
         }
         // acquire: a deletion's tasks need the cores and change stamps as their
         // producers left them (measured necessary: without it, warps running
@@ -937,12 +1055,13 @@ __device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const Ma
         // nothing of a vertex but its per-iteration word, which is only ever
         // read and updated at L2, and its record, which is read with acquire.
         if (DEL || __any_sync(0xffffffffu, t != TASK_EMPTY && (int)(t >> 62) == T_CHUNK)) __threadfence();
-        run_batch<DEL>(g, C, P, B, W, e, ls, t);
+        run_batch<DEL>(g, C, P, B, W, e, e0, t);
         __syncwarp();
         if (look) {
             h = __shfl_sync(0xffffffffu, h, 0);
             tl = __shfl_sync(0xffffffffu, tl, 1);
             const unsigned long long backlog = tl > h ? tl - h : 0ull;
+            const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
             const unsigned long long c = backlog * share / (2 * nwarps);
             claim = c < 1 ? 1 : c > 32 ? 32 : (int)c;
             W.klim = backlog > 2 * nwarps ? 32 : 1;
@@ -967,6 +1086,60 @@ __device__ __forceinline__ void seed_tasks(Ctl* C, const MaintainParams& P, cons
         if (task_room(C, P, tb, cnt) && (unsigned long long)lane < cnt)
             vstore64(&P.TQ[(tb + lane) & P.tqmask],
                      mk_task(type, (unsigned long long)(uint32_t)log[(base + lane) & P.qmask]));
+    }
+}
+
+// ---------------------------------------------------------------- SD fix-up
+// Grid mode's fixup_vertex (cm_vertex.cuh): the SD of a vertex whose core
+// moved in iteration fe, and that of its unmoved neighbours that count it
+// differently now.  Windows of 512 slots as in the search; a group of many
+// warps deals them round robin.  link: iterations follow, so a neighbour at
+// the riser's new level takes it into its record.
+template <int OP, class Grp>
+__device__ __forceinline__ void fixup_wide(const DevGraph& g, const MaintainParams& P, WarpBuf& B, int v, uint32_t fe,
+                                           uint32_t e0, bool link) {
+    const int lane = lane_id();
+    const int kn = g.hc[v].x;
+    const int32_t* list = g.adj + g.off[v];
+    const int len = g.end[v];
+    const int kk = OP == 0 ? kn : kn + 1;   // neighbours whose SD counts v differently now
+    int sd = 0, ne = 0;
+    for (int s = Grp::first() * 16; s < len; s += Grp::G * 16) {
+        const int nc = scan_window<OP == 0 ? S_ROSE : S_DROPPED>(g, list, false, s, len, kk, false, B, sd, ne);
+        for (int b0 = 0; b0 < nc; b0 += 128) {
+            int id[4];
+            uint32_t ch[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int i = b0 + j * 32 + lane;
+                id[j] = i < nc ? B.id[i] : -1;
+                ch[j] = i < nc ? __ldcg(g.chg + id[j]) : fe;
+            }
+            // all of this phase's changes to a neighbour go the same way, so
+            // only the update that crosses its core moves its key bit
+            int old[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                old[j] = ch[j] != fe ? atomicAdd(&g.hc[id[j]].y, OP == 0 ? 1 : -1) : -1;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                if (ch[j] == fe) continue;
+                if (OP == 0) {
+                    if (old[j] == kk) atomicOr(&g.kc[id[j]], 1u);
+                    if (link) rec_link(P, e0, id[j], kk, v, false);
+                } else if (old[j] == kk + 1) {
+                    atomicAnd(&g.kc[id[j]], ~1u);
+                }
+            }
+        }
+        __syncwarp();
+    }
+    sd = Grp::sum(sd);
+    if (Grp::rank0()) {
+        g.hc[v].y = sd;
+        g.kc[v] = key_of(kn, sd);
+        note(B, N_CH, 1);
+        note(B, N_CHL, len);
     }
 }
 

@@ -68,3 +68,38 @@ def test_list_lengths(cm, d, opts):
         assert (g.superior_degrees() == _sd(n, cur, ref)).all(), (d, b)
     assert g.stats()["grid_iterations"] == g.stats()["iterations"] > 0
     g.close()
+
+
+@pytest.mark.parametrize("hub_slots", [1024, 300, -1])
+def test_many_iterations(cm, hub_slots):
+    """A batch whose edges meet at a few vertices takes dozens of iterations in
+    one launch: vertices are searched again from the records that earlier
+    iterations left, which new edges and risen neighbours have joined.
+    Iterations, cores and superior degrees against the oracle."""
+    import torch
+    rng = np.random.default_rng(5)
+    n = 2600
+    # dense blocks of several levels, so that vertices rise into occupied ones
+    p = np.repeat([0.9, 0.6, 0.35, 0.2], n // 4)
+    i, j = np.triu_indices(n, 1)
+    keep = rng.random(len(i)) < p[i] * p[j]
+    e = np.stack([i[keep], j[keep]], 1).astype(np.int32)
+    g = cm.CoreGraph(n, torch.from_numpy(e).cuda(), block_mode_edges=-1, hub_slots=hub_slots)
+    ref = oracle.OracleGraph(n, e, mode=oracle.SUPERIOR)
+    hot = rng.choice(n, 40, replace=False)
+    for b in range(3):
+        x = np.stack([rng.choice(hot, 900), rng.integers(0, n, 900)], 1).astype(np.int32)
+        x = x[x[:, 0] != x[:, 1]]
+        for f, r in ((g.insert_edges, ref.insert_edges), (g.delete_edges, ref.delete_edges)):
+            if b == 2 and f == g.delete_edges:
+                break
+            assert f(torch.from_numpy(x).cuda()) == r(x)
+            st = g.stats()
+            assert st["iterations"] == ref.last_iterations() == st["grid_iterations"]
+            cores = ref.cores()
+            assert (g.cores() == cores).all(), b
+            cur = np.asarray(ref.edges(), dtype=np.int64)
+            cur = np.sort(cur, 1)
+            assert (g.superior_degrees() == _sd(n, cur[:, 0] * n + cur[:, 1], cores)).all(), b
+    assert st["iterations"] > 10
+    g.close()
