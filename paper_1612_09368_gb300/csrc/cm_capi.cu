@@ -929,6 +929,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         h->m -= nrem0;
     } else {
         h->m += nrem0;
+        if (nrem0 > 0) h->idx_tomb -= (int64_t)c.reused;   // read with the call's last status
     }
     h->last.applied += nrem0;
     if (n_applied) *n_applied = nrem0;
@@ -1763,6 +1764,7 @@ static int step_finish(cm_step* s, const long long k[2], int64_t* applied[2]) {
         const long long kept = (long long)L.kept[p];
         if (p == 0) {
             h->idx_live += kept;
+            h->idx_tomb -= (int64_t)c.reused;
             h->m += kept;
         } else {
             h->idx_live -= kept;

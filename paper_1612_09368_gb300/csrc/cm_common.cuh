@@ -142,6 +142,7 @@ struct __align__(128) Ctl {
     unsigned long long adj_top;    // bump pointer of the adjacency pool
     long long bad_index;           // smallest invalid input position
     unsigned long long gather_n;   // gathered incident edges (vertex deletion)
+    unsigned long long reused;     // buckets of deleted keys that the inserted ones took
     int min_deg;                   // peel: smallest remaining degree
     int defer;                     // captured step: skip its remaining kernels (1 pool short, 2 error)
     unsigned long long passes;     // captured step: launch pairs of the current phase
@@ -238,6 +239,29 @@ __device__ __forceinline__ long long idx_insert(Bucket* idx, unsigned long long 
             unsigned long long old = atomicCAS(&idx[b].key, KEY_EMPTY, key);
             if (old == KEY_EMPTY) { *existed = false; return (long long)b; }
             if (old == key) { *existed = true; return (long long)b; }
+        }
+        b = (b + 1) & mask;
+    }
+    return -1;
+}
+
+// Place a key known to be absent (and placed by one thread only) in the
+// first free bucket of its probe sequence, an empty one or one that a deleted
+// key left (*reused).  Taking the latter keeps the sequences short: without
+// it, an edge that comes and goes leaves one dead bucket per round in its own
+// sequence (one edge of a 10^4-vertex graph inserted and deleted 1,000 times:
+// 1.8 ms a pass, against 0.6 on a new graph).  Returns the bucket; -1 if full.
+__device__ __forceinline__ long long idx_place(Bucket* idx, unsigned long long mask, unsigned long long key, bool* reused) {
+    unsigned long long b = fmix64(key) & mask;
+    for (unsigned long long probe = 0; probe <= mask; probe++) {
+        unsigned long long k = idx[b].key;
+        while (k == KEY_EMPTY || k == KEY_TOMB) {   // a lost race leaves another key, or the race for a dead bucket
+            const unsigned long long old = atomicCAS(&idx[b].key, k, key);
+            if (old == k) {
+                *reused = k == KEY_TOMB;
+                return (long long)b;
+            }
+            k = old;
         }
         b = (b + 1) & mask;
     }

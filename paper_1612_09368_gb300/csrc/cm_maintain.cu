@@ -33,6 +33,7 @@ __global__ void ctl_reset_ingest_kernel(Ctl* c) {
     c->reloc_need = 0;
     c->bad_index = 0x7F7F7F7F7F7F7F7FLL;   // larger than any position
     c->gather_n = 0;
+    c->reused = 0;
     c->defer = 0;
 }
 
@@ -148,12 +149,13 @@ __global__ void index_new_edges_kernel(REdge* R, long long n, const unsigned lon
     n = item_count(n, np);
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        bool existed = false;
-        long long bk = idx_insert(g.idx, g.idx_mask, ekey(R[i].lo, R[i].hi), &existed);
-        if (bk < 0 || existed) {
+        bool reused = false;   // ingest kept the edge because the graph lacks it, and once
+        long long bk = idx_place(g.idx, g.idx_mask, ekey(R[i].lo, R[i].hi), &reused);
+        if (bk < 0) {
             atomicCAS(&c->error, 0, E_INDEX_FULL);
             continue;
         }
+        if (reused) atomicAdd(&c->reused, 1ull);
         g.idx[bk].slo = -2;
         g.idx[bk].shi = -2;
         R[i].bkt = (uint32_t)bk;
@@ -304,6 +306,7 @@ __global__ void step_begin_kernel(Ctl* c, StepLog* log) {
     c->reloc_need = 0;
     c->bad_index = 0x7FFFFFFFFFFFFFFFll;
     c->gather_n = 0;
+    c->reused = 0;
     unsigned char* p = reinterpret_cast<unsigned char*>(log);
     for (unsigned i = 0; i < sizeof(StepLog); i++) p[i] = 0;
 }
