@@ -759,36 +759,57 @@ static MaintainParams handle_params(const cm_graph* h, int op) {
 
 // mode 0: maintain cores; mode 1: structure only (cores become stale).
 // per_graph (host, nullable): per-graph kept counts of a multi-graph batch.
+// host_sized: the host reads the counts of ingest and grows the adjacency
+// pool before the lists move (otherwise only when the device finds it short).
 static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, int64_t* n_applied, int mode,
-                         int64_t* per_graph) {
+                         int64_t* per_graph, bool host_sized = false) {
     DevGraph& g = h->g;
     g.n = h->n;
     int rc;
     if (op == CM_OP_INSERT && (rc = ensure_index(h, k))) return rc;
-    // A plain delete needs nothing from ingest on the host before the
-    // maintenance launches (no relocation, no index growth): the kept count
-    // stays on the device, the first launch takes it from there, and an
-    // invalid id stops every kernel after ingest (they test the error word
-    // first) before anything changed.  The host reads the control block
-    // once, at the end.
-    const bool device_count = op == CM_OP_DELETE && mode == 0 && !per_graph;
+    // A plain call needs nothing from ingest on the host before the
+    // maintenance launches: the kept count stays on the device, the first
+    // launch takes it from there, an invalid id stops every kernel after
+    // ingest (they test the error word first) before anything changed, and
+    // so does a pool too short for the lists that must move (Ctl::defer; the
+    // call then starts over with the host in between).  The host reads the
+    // control block once, at the end.
+    const bool hooks = op == CM_OP_INSERT && (h->opt.debug_flags & ~CM_DEBUG_CHECK_ITERATIONS) != 0;
+    const bool device_count = mode == 0 && !per_graph && !host_sized && !hooks;
+    const bool small = device_count && k <= kSmallBatch;
     if (device_count && (rc = ensure_tasks(h))) return rc;
-    CK(h, cudaMemsetAsync(h->bset, 0xFF, h->bset_size * sizeof(BSet), h->stream));
-    LAUNCH(h, ctl_reset_ingest(h->ctl, h->stream));
-    LAUNCH(h, ingest_a(dE, k, nullptr, g, h->bset, h->bset_size - 1, h->ctl, h->stream));
-    LAUNCH(h, ingest_b(dE, k, nullptr, op, g, h->bset, h->bset_size - 1, h->R0, h->OVL, h->ctl, h->stream));
+    if (mode == 0 && h->epoch > 0x3F000000u) {   // 30-bit stamps about to wrap: clear them
+        CK(h, cudaMemsetAsync(g.chg, 0, (size_t)h->n * 4, h->stream));
+        CK(h, cudaMemsetAsync(g.taken, 0, (size_t)h->n * 4, h->stream));
+        CK(h, cudaMemsetAsync(g.hw, 0, (size_t)h->n * sizeof(unsigned long long), h->stream));
+        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, h->stream));
+        h->epoch = 1;
+    }
+    // where the iterations start: all kept edges remain, in R0.  Every call
+    // starts grid-wide: even one edge can start a search over a whole dense
+    // shell; the kernel hands down after a small iteration.
+    Resume rs{};
+    rs.epoch = h->epoch;
     Ctl& c = *h->hctl;
     long long nrem0 = k;   // an upper bound until the count is read
-    if (!device_count) {
-        if ((rc = rd_ctl(h))) return rc;
-        if (c.error == E_INVALID)
-            return set_err(h, CM_ERR_INVALID, "edge %lld of the batch names a vertex out of range or deleted",
-                           c.bad_index);
-        if (c.error) {
-            h->poisoned = true;
-            return set_err(h, CM_ERR_CUDA, "device error %d during ingest", c.error);
+    if (small) {
+        LAUNCH(h, ingest_small(dE, (int)k, op, g, h->R0, h->ctl, rs, h->stream));
+    } else {
+        CK(h, cudaMemsetAsync(h->bset, 0xFF, h->bset_size * sizeof(BSet), h->stream));
+        LAUNCH(h, ctl_reset_ingest(h->ctl, h->stream));
+        LAUNCH(h, ingest_a(dE, k, nullptr, g, h->bset, h->bset_size - 1, h->ctl, h->stream));
+        LAUNCH(h, ingest_b(dE, k, nullptr, op, g, h->bset, h->bset_size - 1, h->R0, h->OVL, h->ctl, h->stream));
+        if (!device_count) {
+            if ((rc = rd_ctl(h))) return rc;
+            if (c.error == E_INVALID)
+                return set_err(h, CM_ERR_INVALID, "edge %lld of the batch names a vertex out of range or deleted",
+                               c.bad_index);
+            if (c.error) {
+                h->poisoned = true;
+                return set_err(h, CM_ERR_CUDA, "device error %d during ingest", c.error);
+            }
+            nrem0 = (long long)c.nrem;
         }
-        nrem0 = (long long)c.nrem;
     }
     if (per_graph && h->dpergraph) {
         CK(h, cudaMemsetAsync(h->dpergraph, 0, (size_t)h->ngraphs * 8, h->stream));
@@ -796,7 +817,16 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         CK(h, cudaMemcpyAsync(per_graph, h->dpergraph, (size_t)h->ngraphs * 8, cudaMemcpyDeviceToHost, h->stream));
         CK(h, cudaStreamSynchronize(h->stream));
     }
-    if (op == CM_OP_INSERT) {
+    if (small) {
+        // ingest_small has placed the new edges
+    } else if (op == CM_OP_INSERT && device_count) {
+        const unsigned long long *kept = &h->ctl->nrem, *over = &h->ctl->noverflow;
+        LAUNCH(h, reloc_size(h->OVL, 2 * k, over, g, h->ctl, h->stream));
+        LAUNCH(h, insert_gate(g, h->ctl, h->stream));
+        LAUNCH(h, relocate(h->OVL, 2 * k, over, g, h->ctl, h->stream));
+        LAUNCH(h, index_new_edges(h->R0, k, kept, g, h->ctl, h->stream));
+        LAUNCH(h, clear_need(h->R0, k, kept, g, h->stream));
+    } else if (op == CM_OP_INSERT) {
         // Device memory the call may still need comes first: up to here
         // ingest only counted pending insertions (need[]), so a failed
         // allocation clears them and leaves the graph as it was.
@@ -817,7 +847,6 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         // relocation moves lists without changing the graph
         if (mode == 0 && nrem0 > 0 && (rc = ensure_tasks(h))) return undo_need(rc);
         if (novl > 0) LAUNCH(h, relocate(h->OVL, novl, nullptr, h->g, h->ctl, h->stream));
-        h->idx_live += nrem0;
         LAUNCH(h, index_new_edges(h->R0, nrem0, nullptr, h->g, h->ctl, h->stream));
         LAUNCH(h, clear_need(h->R0, nrem0, nullptr, h->g, h->stream));
     } else if (mode == 0 && nrem0 > 0 && (rc = ensure_tasks(h))) {
@@ -831,13 +860,6 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
             return set_err(h, CM_ERR_LIMIT, "structure update failed with device error %d", c.error);
         }
     } else if (nrem0 > 0) {
-        if (h->epoch > 0x3F000000u) {   // 30-bit stamps about to wrap: clear them
-            CK(h, cudaMemsetAsync(g.chg, 0, (size_t)h->n * 4, h->stream));
-            CK(h, cudaMemsetAsync(g.taken, 0, (size_t)h->n * 4, h->stream));
-            CK(h, cudaMemsetAsync(g.hw, 0, (size_t)h->n * sizeof(unsigned long long), h->stream));
-            CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, h->stream));
-            h->epoch = 1;
-        }
         MaintainParams p = handle_params(h, op);
         p.max_iters = nrem0 + 1;
         int blocks, threads;
@@ -861,17 +883,10 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         // debug mode: one iteration per launch pair, the store checked after each
         const bool check_each = (h->opt.debug_flags & CM_DEBUG_CHECK_ITERATIONS) != 0;
         p.yield_each = check_each ? 1 : 0;
-        // where the call starts: all kept edges remain, in R0
-        Resume rs{};
-        rs.nrem = (unsigned long long)nrem0;   // replaced on the device by ingest's count (device_count)
-        rs.rsel = 0;
-        rs.epoch = h->epoch;
-        rs.done = 0;
-        // every call starts grid-wide: even one edge can start a search over a
-        // whole dense shell; the kernel hands down after a small iteration
-        rs.want = 0;
-        rs.iters = 0;
-        LAUNCH(h, ctl_begin_maintain(h->ctl, rs, device_count ? 1 : 0, h->stream));
+        if (!small) {
+            rs.nrem = (unsigned long long)nrem0;   // replaced on the device by ingest's count (device_count)
+            LAUNCH(h, ctl_begin_maintain(h->ctl, rs, device_count ? 1 : 0, h->stream));
+        }
         CK(h, cudaEventRecord(h->ev[2], h->stream));
         // grid launch then block launch: whichever the resume state names runs,
         // the other returns at once; a handover inside the pair needs no host.
@@ -882,7 +897,8 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
                 return set_err(h, CM_ERR_LIMIT, "maintenance did not finish within %d launch pairs", pass);
             }
             if (want_grid) LAUNCH(h, launch_maintain(p, blocks, threads, h->stream));
-            LAUNCH(h, launch_maintain_block(p, h->stream));
+            // (one edge is one iteration, and a call's first is grid-wide: nothing to hand over)
+            if (!(want_grid && pass == 0 && nrem0 == 1)) LAUNCH(h, launch_maintain_block(p, h->stream));
             if ((rc = rd_ctl(h))) return rc;
             if (check_each && !c.error) {
                 cm_check_report r{};
@@ -905,6 +921,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
             if (c.error == E_INVALID)
                 return set_err(h, CM_ERR_INVALID, "edge %lld of the batch names a vertex out of range or deleted",
                                c.bad_index);
+            if (c.defer && !c.error) return update_device(h, op, dE, k, n_applied, mode, per_graph, true);
             nrem0 = (long long)c.nrem;
         }
         if (c.error) {
@@ -929,6 +946,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         h->m -= nrem0;
     } else {
         h->m += nrem0;
+        h->idx_live += nrem0;
         if (nrem0 > 0) h->idx_tomb -= (int64_t)c.reused;   // read with the call's last status
     }
     h->last.applied += nrem0;

@@ -76,8 +76,13 @@ cudaError_t index_new_edges(REdge* R, long long n, const unsigned long long* np,
 cudaError_t reloc_size(const int32_t* ovl, long long novl, const unsigned long long* np, DevGraph g, Ctl* c,
                        cudaStream_t s);
 cudaError_t reloc_gate(DevGraph g, Ctl* c, StepLog* log, int phase, cudaStream_t s);
+cudaError_t insert_gate(DevGraph g, Ctl* c, cudaStream_t s);
 cudaError_t relocate(const int32_t* ovl, long long novl, const unsigned long long* np, DevGraph g, Ctl* c,
                      cudaStream_t s);
+// all of the above and ctl_begin_maintain for k <= kSmallBatch edges, in one launch
+constexpr int kSmallBatch = 1024;
+cudaError_t ingest_small(const int32_t* E, int k, int op, DevGraph g, REdge* R0, Ctl* c, const Resume& rs,
+                         cudaStream_t s);
 cudaError_t clear_need(const REdge* R, long long n, const unsigned long long* np, DevGraph g, cudaStream_t s);
 cudaError_t step_begin(Ctl* c, StepLog* log, cudaStream_t s);
 cudaError_t phase_begin(Ctl* c, StepLog* log, int phase, cudaStream_t s);
