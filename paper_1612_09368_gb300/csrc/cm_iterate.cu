@@ -403,7 +403,16 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         remsum += (long long)nrem;
         // ------------------------------------------------ SELECT
         int r = 0;
-        for (;;) {
+        const bool lone = nrem == 1 && !fx;
+        if (lone) {   // one edge is the maximal set: no claim, no barrier (this thread applies it, too)
+            if (MODE == 0) reset_tasks();
+            if (leader) {
+                Rc[0].flags = F_SEL;
+                ls.sel++;
+            }
+            r = 1;
+        }
+        while (!lone) {
             if (r == 0 && fx) {
                 for_each_vertex<MODE>(g, P, &C->pc[2], FXQ, qm, fx_lo, fx_hi, fixup_body);
                 fx = false;
