@@ -457,14 +457,13 @@ static bool check_clean(const cm_check_report& r);
 // Builds the store from a device edge list (global ids).
 static int build_store(cm_graph* h, const int32_t* dE, long long m, const int32_t* dcores) {
     DevGraph& g = h->g;
-    uint32_t* ebkt = (uint32_t*)dalloc(h, (size_t)(m > 0 ? m : 1) * sizeof(uint32_t));
-    if (!ebkt) return set_err(h, CM_ERR_OOM, "out of device memory (create)");
+    int2* at = (int2*)dalloc(h, (size_t)(m > 0 ? m : 1) * sizeof(int2));   // each edge's slots in its two lists
+    if (!at) return set_err(h, CM_ERR_OOM, "out of device memory (create)");
     int rc = CM_OK;
     do {
         if ((rc = reset_ingest_zone(h))) break;
-        h->launches += 3;
-        cudaError_t e = build_index(dE, m, g, ebkt, h->ctl, h->stream);
-        if (e == cudaSuccess) e = count_degrees(dE, ebkt, m, g, h->stream);
+        h->launches += 2;
+        cudaError_t e = build_index(dE, m, g, at, h->ctl, h->stream);
         if (e == cudaSuccess) e = sum_caps(g, 0, g.n, h->ctl, h->stream);
         if (e != cudaSuccess) { rc = fail_cuda(h, e, "build"); break; }
         if ((rc = rd_ctl(h))) break;
@@ -476,6 +475,7 @@ static int build_store(cm_graph* h, const int32_t* dE, long long m, const int32_
             rc = set_err(h, CM_ERR_CUDA, "device error %d while building the index", h->hctl->error);
             break;
         }
+        h->m = (int64_t)h->hctl->nrem;   // edges kept
         long long total = (long long)h->hctl->reloc_need;
         long long pool = total + total / 4 + 4096;
         g.adj = (int32_t*)dalloc(h, (size_t)pool * sizeof(int32_t));
@@ -484,7 +484,7 @@ static int build_store(cm_graph* h, const int32_t* dE, long long m, const int32_
         if ((e = cudaMemsetAsync(&h->ctl->adj_top, 0, 8, h->stream)) != cudaSuccess) { rc = fail_cuda(h, e, "memset"); break; }
         h->launches += 2;
         e = assign_offsets(g, 0, g.n, h->ctl, h->stream);
-        if (e == cudaSuccess) e = scatter_edges(dE, ebkt, m, g, h->stream);
+        if (e == cudaSuccess) e = scatter_edges(dE, at, m, g, h->stream);
         if (e != cudaSuccess) { rc = fail_cuda(h, e, "scatter"); break; }
         if (dcores) {
             h->launches++;
@@ -497,17 +497,8 @@ static int build_store(cm_graph* h, const int32_t* dE, long long m, const int32_
         if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) { rc = fail_cuda(h, e, "create"); break; }
     } while (0);
     cudaStreamSynchronize(h->stream);
-    dfree(h, ebkt, (size_t)(m > 0 ? m : 1) * sizeof(uint32_t));
+    dfree(h, at, (size_t)(m > 0 ? m : 1) * sizeof(int2));
     return rc;
-}
-
-static int count_live_edges(cm_graph* h, long long* m) {
-    std::vector<int32_t> deg((size_t)h->n);
-    if (h->n) CK(h, cudaMemcpy(deg.data(), h->g.deg, (size_t)h->n * 4, cudaMemcpyDeviceToHost));
-    long long s = 0;
-    for (int32_t d : deg) s += d;
-    *m = s / 2;
-    return CM_OK;
 }
 
 // Creates a handle around n vertices and a DEVICE-or-host edge list.
@@ -577,10 +568,7 @@ static int create_common(int32_t n, const int32_t* edges, long long m, const int
     dfree(h, tmp, (size_t)m * 8);
     dfree(h, tmpc, (size_t)(n > 0 ? n : 1) * 4);
     if (rc) return rc;
-    long long live = 0;
-    if ((rc = count_live_edges(h, &live))) return rc;
-    h->m = live;
-    h->idx_live = live;
+    h->idx_live = h->m;
     h->bases = {0, n};
     return CM_OK;
 }

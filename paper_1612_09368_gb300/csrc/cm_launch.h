@@ -94,10 +94,9 @@ cudaError_t launch_maintain_block(const MaintainParams& p, cudaStream_t s);
 int maintain_blocks_per_sm(int threads);
 
 // ---- store / peel (cm_store.cu)
-cudaError_t build_index(const int32_t* E, long long m, DevGraph g, uint32_t* ebkt, Ctl* c, cudaStream_t s);
-cudaError_t count_degrees(const int32_t* E, const uint32_t* ebkt, long long m, DevGraph g, cudaStream_t s);
+cudaError_t build_index(const int32_t* E, long long m, DevGraph g, int2* at, Ctl* c, cudaStream_t s);
 cudaError_t assign_offsets(DevGraph g, int32_t v0, int32_t v1, Ctl* c, cudaStream_t s);
-cudaError_t scatter_edges(const int32_t* E, const uint32_t* ebkt, long long m, DevGraph g, cudaStream_t s);
+cudaError_t scatter_edges(const int32_t* E, const int2* at, long long m, DevGraph g, cudaStream_t s);
 cudaError_t set_cores(const int32_t* cores, DevGraph g, cudaStream_t s);
 // core_scratch: n int32 of scratch (receives a compact copy of the cores)
 cudaError_t init_mcd(DevGraph g, int32_t v0, int32_t v1, int32_t* core_scratch, cudaStream_t s);
