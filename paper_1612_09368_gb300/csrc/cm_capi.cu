@@ -492,8 +492,8 @@ static int build_store(cm_graph* h, const int32_t* dE, long long m, const int32_
         } else {
             if ((rc = peel_all(h))) break;
         }
-        h->launches += 2;
-        if ((e = init_mcd(g, 0, g.n, h->CQ, h->stream)) != cudaSuccess) { rc = fail_cuda(h, e, "init_mcd"); break; }
+        h->launches += 3;
+        if ((e = init_mcd(g, 0, g.n, h->CQ, h->VQ, h->ctl, h->stream)) != cudaSuccess) { rc = fail_cuda(h, e, "init_mcd"); break; }
         if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) { rc = fail_cuda(h, e, "create"); break; }
     } while (0);
     cudaStreamSynchronize(h->stream);
@@ -664,8 +664,8 @@ extern "C" int cm_recompute_cores(cm_graph* h) {
     if ((rc = peel_all(h))) return end_call(h, rc);
     DevGraph g = h->g;
     g.n = h->n;
-    h->launches++;   // init_mcd launches two kernels
-    LAUNCH(h, init_mcd(g, 0, h->n, h->CQ, h->stream));   // CQ holds >= n entries
+    h->launches += 2;   // init_mcd launches three kernels
+    LAUNCH(h, init_mcd(g, 0, h->n, h->CQ, h->VQ, h->ctl, h->stream));   // the rings hold >= n entries
     CK(h, cudaEventRecord(h->ev[3], h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     float ms = 0;

@@ -98,8 +98,9 @@ cudaError_t build_index(const int32_t* E, long long m, DevGraph g, int2* at, Ctl
 cudaError_t assign_offsets(DevGraph g, int32_t v0, int32_t v1, Ctl* c, cudaStream_t s);
 cudaError_t scatter_edges(const int32_t* E, const int2* at, long long m, DevGraph g, cudaStream_t s);
 cudaError_t set_cores(const int32_t* cores, DevGraph g, cudaStream_t s);
-// core_scratch: n int32 of scratch (receives a compact copy of the cores)
-cudaError_t init_mcd(DevGraph g, int32_t v0, int32_t v1, int32_t* core_scratch, cudaStream_t s);
+// core_scratch, hub_scratch: n int32 of scratch each (a compact copy of the cores; vertices with long lists)
+cudaError_t init_mcd(DevGraph g, int32_t v0, int32_t v1, int32_t* core_scratch, int32_t* hub_scratch, Ctl* c,
+                     cudaStream_t s);
 cudaError_t launch_peel(const PeelParams& p, int blocks, cudaStream_t s);
 cudaError_t rehash(const Bucket* old_idx, unsigned long long old_size, DevGraph g, Ctl* c, cudaStream_t s);
 cudaError_t validate_vertices(const int64_t* nbr_off, const int32_t* nbrs, int32_t count, int32_t base, DevGraph g,

@@ -1,4 +1,4 @@
-"""The full decomposition where its paths meet: cascades longer than a block
+"""The full decomposition, and the superior degrees computed after it, where their paths meet: cascades longer than a block
 follows alone (paths, grids), more departures at once than a block's queue
 holds (forests, stars), lists long enough to be shared in chunks, empty
 levels, and lists that start anywhere in a caller's CSR.  Exact comparison
@@ -62,6 +62,13 @@ def _graph(kind):
     return 1, np.zeros((0, 2), np.int32)
 
 
+def _sd(n, e, cores):
+    """Neighbours with a core of at least the vertex's own; -1 for a dead vertex."""
+    cu, cv = cores[e[:, 0]], cores[e[:, 1]]
+    sd = np.bincount(e[:, 0][cv >= cu], minlength=n) + np.bincount(e[:, 1][cu >= cv], minlength=n)
+    return np.where(cores < 0, -1, sd)
+
+
 KINDS = ["path", "cycle-with-tail", "stars", "tree", "cliques", "bipartite", "grid", "rmat", "31-vertices", "single"]
 
 
@@ -72,8 +79,10 @@ def test_store(cm, kind):
     ref = oracle.bz(n, e)
     g = cm.CoreGraph(n, torch.from_numpy(e).cuda() if len(e) else e)
     assert (g.cores() == ref).all()
+    assert (g.superior_degrees() == _sd(n, e, ref)).all()
     g.recompute_cores()
     assert (g.cores() == ref).all()
+    assert (g.superior_degrees() == _sd(n, e, ref)).all()
     if n > 100:   # holes in the lists, dead vertices
         dead = np.arange(0, n, 97, dtype=np.int32)
         g.delete_vertices(dead)
@@ -84,6 +93,7 @@ def test_store(cm, kind):
         g.apply_edges(cm.CM_OP_INSERT, e[live][:50])
         g.recompute_cores()
         assert (g.cores() == want).all()
+        assert (g.superior_degrees() == _sd(n, e[live], want)).all()
     g.close()
 
 
