@@ -50,7 +50,7 @@ def load_peaks():
         return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("cm_iterate.cu", "cm_vertex.cuh", "cm_common.cuh", "cm_launch.h")
+KERNEL_SOURCES = ("cm_iterate.cu", "cm_search.cuh", "cm_vertex.cuh", "cm_common.cuh", "cm_launch.h")
 
 
 def _code_only(src: str) -> str:

@@ -67,7 +67,7 @@ typedef void (*cm_free_fn)(void* ptr, size_t bytes, void* stream, void* ctx);
 typedef struct cm_options {
     int32_t slack_pct;      /* per-vertex adjacency headroom in percent (default 25) */
     int32_t min_cap;        /* minimum adjacency slots per vertex, rounded up to 4 (default 4) */
-    int32_t block_threads;  /* unused (kept for layout): every persistent kernel runs 512-thread blocks */
+    int32_t block_threads;  /* unused (kept for layout): every persistent kernel has its own block size */
     int32_t blocks_per_sm;  /* resident blocks per SM of the persistent kernels; 0 = occupancy limit */
     int32_t max_sms;        /* SMs the persistent kernels may fill; 0 = all (lower it to share the GPU) */
     int32_t block_mode_edges; /* single-block mode only while at most this many edges remain (16384;
@@ -81,9 +81,9 @@ typedef struct cm_options {
     int32_t block_mode_leave; /* single block -> grid after an iteration touching more (8192) */
     int32_t hub_slots;      /* grid mode: a vertex with at least this many adjacency slots is scanned by
                                all warps in chunks of 512 (1024; negative = never) */
-    int32_t block_slots;    /* grid mode, insert: outside the search, a vertex with at least this many slots
-                               is scanned by a whole block instead of one warp (4096, the least that counts) */
-    int32_t block_slots_delete; /* the same for delete calls (values below 4096 count as 4096) */
+    int32_t block_slots;    /* grid mode, insert: outside the search, a list of more than 256 slots is scanned
+                               by several warps, this many slots each (4096; rounded down to 512 slots) */
+    int32_t block_slots_delete; /* the same for delete calls (1024) */
     int32_t task_claim;     /* grid mode: multiple of its fair share of the waiting search tasks that a warp
                                claims at once (1..8, default 1) */
     int32_t select_order;   /* order of the greedy superior-edge-set selection (Section IV,
@@ -334,8 +334,9 @@ typedef struct cm_step_config {
     int32_t block_mode_enter;
     int32_t block_mode_leave;
     int32_t hub_slots;         /* frontier granularity: grid-wide chunked scans from this many slots (0 = 1024, -1 never) */
-    int32_t blocks_per_sm;     /* block shape of the grid-mode launch: resident 512-thread blocks per SM (0 = max) */
-    int32_t block_slots;       /* frontier granularity: block-wide scans from this many slots, insert phase (0 = 4096) */
+    int32_t blocks_per_sm;     /* block shape of the grid-mode launch: resident blocks per SM (0 = max) */
+    int32_t block_slots;       /* granularity outside the search: slots a warp scans of a long list, insert phase
+                                  (0 = 4096) */
     int32_t task_claim;        /* multiple of its fair share of the waiting search tasks that a warp claims (0 = 1) */
     int32_t reserved;
 } cm_step_config;
@@ -462,7 +463,7 @@ void cm_server_destroy(cm_server* s);
  * in both endpoints' rows).  cores (device, n int32) receives the result.
  * Runs on `stream` (cudaStream_t) and returns after completion.  It
  * allocates nothing: its scratch is one static device array sized for at
- * most 1,048,576 vertices (16 MiB, plus 2 MiB of chunk tasks for the lists
+ * most 1,048,576 vertices (12 MiB, plus 2 MiB of chunk tasks for the lists
  * of high-degree vertices and a 4 KiB control block), held by every
  * GPU that loads the library until the process exits.  All calls share that
  * array: calls whose work overlaps on the GPU (for example on two streams)

@@ -3,9 +3,11 @@
 // A handle owns one graph (or a disjoint union of many) in device memory
 // and runs every call on its stream.  An update call is:
 //   copy batch in -> ingest (validate, canonicalise, dedupe, filter against
-//   the edge index) -> read back counts -> relocate vertices whose slack the
-//   batch exceeds -> one cooperative launch of the maintenance kernel, which
-//   runs all superior-edge-set iterations -> read back status and counters.
+//   the edge index) -> relocate vertices whose slack the batch exceeds ->
+//   launches of the maintenance kernel, which run all superior-edge-set
+//   iterations -> read back status and counters.  The counts stay on the
+//   device in between; the host steps in only when the adjacency pool is
+//   short (update_device).
 #include <algorithm>
 #include <climits>
 #include <cstdarg>

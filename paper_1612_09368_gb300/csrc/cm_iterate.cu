@@ -55,10 +55,9 @@
 //
 // The per-vertex bodies and the per-iteration vertex word are in cm_vertex.cuh.
 //
-// Per-vertex work of a wave is done by one warp per vertex (vertices fetched
-// dynamically); a vertex with at least P.block_len adjacency slots (256 in
-// single-block mode) is deferred
-// and then processed by the whole block of the warp that fetched it.
+// In single-block mode a wave's vertices get one warp each (fetched
+// dynamically); one with at least 256 slots is deferred and then processed by
+// the whole block.  The grid's searches and fix-ups are in cm_search.cuh.
 #include <type_traits>
 
 #include "cm_common.cuh"
@@ -79,15 +78,10 @@ constexpr int kGridThreads = 384;
 static_assert(kGridThreads / 32 == kGridWarps, "one search buffer per grid-mode warp");
 constexpr int kMaxBig = 64;
 constexpr int kBlockLenSingle = 256;   // single-block mode: the block scans lists from this size
-// Grid mode: never below this, whatever the options say.  A warp walks 512
-// slots a step, so a block on a shorter list leaves most of its warps idle
-// (10^6 degree-proportional deletes on R-MAT scale 24, 1024 -> 4096: 30.3 ->
-// 26.9 ms).
-constexpr int kBlockLenGrid = 4096;
 
-// The iteration loop's state while a grid-wide search runs.
+// The iteration loop's state while a grid-wide search or fix-up runs.
 struct LoopState {
-    unsigned long long nrem, nrem_next, vq0, eq0, cq0, vq_t, eq_t, cq_t;
+    unsigned long long nrem, nrem_next, vq0, eq0, cq0, vq_t, eq_t, cq_t, fx_lo, fx_hi, fx_long;
     REdge *Rc, *Rn;
     unsigned long long t_last;
     long long remsum, iters0;
@@ -115,33 +109,29 @@ struct Barrier {
 };
 
 // ---------------------------------------------------------------- vertex loop (waves)
-// Runs body(v, Group) for every vertex of ring[lo, hi): one warp per vertex.
-// Each warp's first vertex is dealt by its warp index; the rest are fetched
-// dynamically (counter *ctr, zeroed at every barrier), so a phase with no
-// more vertices than warps touches no shared counter, and a larger one does
-// not start with every warp of the grid at the same counter.  A vertex
-// with at least P.block_len slots (kBlockLenGrid at least; kBlockLenSingle in
-// single-block mode) is deferred by the warp that fetched it and then processed by that warp's
-// whole block, so a long list does not hold a wave on one warp.  Every
-// thread of the launch must call it.
-template <int MODE, class Body>
-__device__ __forceinline__ void for_each_vertex(const DevGraph& g, const MaintainParams& P, unsigned long long* ctr,
-                                                const int32_t* ring, unsigned long long qm, unsigned long long lo,
-                                                unsigned long long hi, Body body) {
-    constexpr int NT = MODE == 0 ? kGridThreads : kBlockThreads;
+// Single-block mode: runs body(v, Group) for every vertex of ring[lo, hi),
+// one warp per vertex.  Each warp's first vertex is dealt by its warp index;
+// the rest are fetched dynamically (counter *ctr, zeroed at every barrier).
+// A vertex with at least kBlockLenSingle slots is deferred by the warp that
+// fetched it and then processed by the whole block, so a long list does not
+// hold a wave on one warp.  Every thread of the launch must call it.
+template <class Body>
+__device__ __forceinline__ void for_each_vertex(const DevGraph& g, unsigned long long* ctr, const int32_t* ring,
+                                                unsigned long long qm, unsigned long long lo, unsigned long long hi,
+                                                Body body) {
     const int lane = lane_id();
     __shared__ int s_big[kMaxBig];
     __shared__ int s_nbig;
     if (threadIdx.x == 0) s_nbig = 0;
     __syncthreads();
-    const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+    constexpr unsigned nw = kBlockThreads / 32;
     const unsigned long long cnt = hi - lo;
-    unsigned long long j = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    unsigned long long j = threadIdx.x >> 5;
     for (;;) {
         if (j >= cnt) break;
         const int v = ring[(lo + j) & qm];
         int defer = 0;
-        if (lane == 0 && g.end[v] >= (MODE == 0 ? max(P.block_len, kBlockLenGrid) : kBlockLenSingle)) {
+        if (lane == 0 && g.end[v] >= kBlockLenSingle) {
             int s = atomicAdd(&s_nbig, 1);
             if (s < kMaxBig) {
                 s_big[s] = v;
@@ -156,7 +146,7 @@ __device__ __forceinline__ void for_each_vertex(const DevGraph& g, const Maintai
     __syncthreads();
     const int nb = min(s_nbig, kMaxBig);
     for (int b = 0; b < nb; b++) {
-        body(s_big[b], BlockGroup<NT>{});
+        body(s_big[b], BlockGroup<kBlockThreads>{});
         __syncthreads();
     }
 }
@@ -342,53 +332,81 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
     // pending SD fix-up of the previous iteration
     bool fx = false;
     unsigned long long fx_lo = 0, fx_hi = 0;
-    uint32_t fx_e = 0;
     // a call whose ingest kept no edge (its count read on the device) is done at once
     int next_want = MODE, finished = (!mid && nrem == 0) ? 1 : 0;
     const int32_t* FXQ = OP == 0 ? P.CQ : P.EQ;
-    auto fixup_body = [&](int v, auto grp) {
-        if constexpr (MODE == 0)
-            fixup_wide<OP, decltype(grp)>(g, P, reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5], v, fx_e, e0,
-                                          nrem > 0);
-        else
-            fixup_vertex<decltype(grp)>(g, v, fx_e, OP, ls);
-    };
+    [[maybe_unused]] unsigned long long fx_long = 0;   // insert: chunks of long lists queued for it; delete: hubs met
 
-    // The grid-wide search, with the loop's state parked in shared memory
-    // meanwhile (every thread holds the same values): see flush_stats.
+    // Runs a grid-wide search or fix-up with the loop's state parked in shared
+    // memory meanwhile (every thread holds the same values): see flush_stats.
+    [[maybe_unused]] auto parked = [&](auto work) {
+        WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
+        flush_stats(B, ls);
+        __shared__ LoopState S;
+        __syncthreads();   // the last reader of S is done
+        if (threadIdx.x == 0) {
+            S = LoopState{nrem, nrem_next, vq0, eq0, cq0, vq_t, eq_t, cq_t, fx_lo, fx_hi, fx_long, Rc, Rn, sync.t_last,
+                          remsum, iters0, e, e0, iters, rounds, waves};
+            s_search_t0 = gtimer();
+        }
+        __syncthreads();
+        const bool fine = work(S);
+        nrem = S.nrem;
+        nrem_next = S.nrem_next;
+        vq0 = S.vq0;
+        eq0 = S.eq0;
+        cq0 = S.cq0;
+        vq_t = S.vq_t;
+        eq_t = S.eq_t;
+        cq_t = S.cq_t;
+        Rc = S.Rc;
+        Rn = S.Rn;
+        sync.t_last = S.t_last;
+        remsum = S.remsum;
+        iters0 = S.iters0;
+        e = S.e;
+        e0 = S.e0;
+        iters = S.iters;
+        rounds = S.rounds;
+        waves = S.waves;
+        return fine;
+    };
     [[maybe_unused]] auto search = [&](auto del) {
         if constexpr (MODE == 0) {
-            WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
-            flush_stats(B, ls);
-            __shared__ LoopState S;
-            __syncthreads();   // the last reader of S is done
-            if (threadIdx.x == 0) {
-                S = LoopState{nrem, nrem_next, vq0, eq0, cq0, vq_t, eq_t, cq_t, Rc, Rn, sync.t_last, remsum, iters0,
-                              e, e0, iters, rounds, waves};
-                s_search_t0 = gtimer();
-            }
-            __syncthreads();
-            const bool fine = async_search<decltype(del)::value>(g, C, P, S.e, S.e0, OP == 0 && S.nrem_next > 0);
-            nrem = S.nrem;
-            nrem_next = S.nrem_next;
-            vq0 = S.vq0;
-            eq0 = S.eq0;
-            cq0 = S.cq0;
-            vq_t = S.vq_t;
-            eq_t = S.eq_t;
-            cq_t = S.cq_t;
-            Rc = S.Rc;
-            Rn = S.Rn;
-            sync.t_last = S.t_last;
-            remsum = S.remsum;
-            iters0 = S.iters0;
-            e = S.e;
-            e0 = S.e0;
-            iters = S.iters;
-            rounds = S.rounds;
-            waves = S.waves;
-            return fine;
+            return parked([&](const LoopState& S) {
+                return async_search<decltype(del)::value>(g, C, P, S.e, S.e0, OP == 0 && S.nrem_next > 0);
+            });
         } else {
+            return true;
+        }
+    };
+    // the pending SD fix-up; false: a barrier failed
+    auto fixup = [&]() {
+        if constexpr (MODE == 0) {
+            // An insertion queues the chunks of long lists as it commits; a
+            // deletion here, at the price of a barrier (~4 us), if its search
+            // met a hub or the vertices are many: with the line at one a warp
+            // R-MAT scale 20 deletions of 10^4 edges took 0.19 ms, not 0.185.
+            bool queued = true;
+            if (OP == 1) {
+                queued = fx_long > 0 || fx_hi - fx_lo > 8ull * (unsigned long long)nwarps;
+                fx_long = 0;
+                if (queued) {
+                    for (unsigned long long i = fx_lo + gwarp * 32 + lane; i < fx_hi; i += nwarps * 32) {
+                        const int v = __ldcg(FXQ + (i & qm));
+                        list_long(g, C, P, v, g.end[v]);
+                    }
+                    if (!sync(PH_FIXUP)) return false;
+                    fx_long = vload64(&C->spc[2]);
+                }
+            }
+            return parked([&](const LoopState& S) {
+                fixup_grid<OP>(g, C, P, FXQ, S.fx_lo, S.fx_hi, queued, S.fx_long, S.e - 1, S.e0, S.nrem > 0);
+                return true;
+            });
+        } else {
+            for_each_vertex(g, &C->pc[2], FXQ, qm, fx_lo, fx_hi,
+                            [&](int v, auto grp) { fixup_vertex<decltype(grp)>(g, v, e - 1, OP, ls); });
             return true;
         }
     };
@@ -414,7 +432,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         }
         while (!lone) {
             if (r == 0 && fx) {
-                for_each_vertex<MODE>(g, P, &C->pc[2], FXQ, qm, fx_lo, fx_hi, fixup_body);
+                if (!(ok = fixup())) break;
                 fx = false;
             }
             if (MODE == 0 && r == 0) reset_tasks();   // nobody pushes tasks before APPLY
@@ -554,10 +572,10 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                         break;
                     }
                     waves++;
-                    for_each_vertex<MODE>(g, P, &C->pc[2], P.VQ, qm, flo, fhi, [&](int v, auto grp) {
+                    for_each_vertex(g, &C->pc[2], P.VQ, qm, flo, fhi, [&](int v, auto grp) {
                         process_frontier<decltype(grp)>(g, C, P, v, load_vinfo(g, v), e, ls);
                     });
-                    for_each_vertex<MODE>(g, P, &C->pc[3], P.EQ, qm, elo, ehi, [&](int v, auto grp) {
+                    for_each_vertex(g, &C->pc[3], P.EQ, qm, elo, ehi, [&](int v, auto grp) {
                         evict_insert_vertex<decltype(grp)>(g, C, P, load_vinfo(g, v), e, ls);
                     });
                     if (!(ok = sync(PH_DISCOVER))) break;
@@ -574,12 +592,13 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             for (long long base = gwarp * 32; base < (long long)(vq_t - vq0); base += nwarps * 32) {
                 long long i = base + lane;
                 bool up = false;
-                int v = 0;
+                int v = 0, len = 0;
                 if (i < (long long)(vq_t - vq0)) {
                     v = P.VQ[(vq0 + i) & qm];
                     const int core = g.hc[v].x;
                     const int support = ww(g.hw[v]);
                     if (support > core) {
+                        if (MODE == 0) len = g.end[v];
                         g.hc[v].x = core + 1;
                         g.kc[v] = key_of(core + 1, 0);   // bit set by the SD fix-up
                         g.chg[v] = e;
@@ -587,8 +606,10 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                     }
                 }
                 warp_push(&C->tail[2], P.CQ, qm, up, v);
+                if constexpr (MODE == 0) list_long(g, C, P, v, len);
             }
             if (!(ok = sync(PH_COMMIT))) break;
+            fx_long = vload64(&C->spc[2]);
             cq_t = vload64(&C->stail[2]);
             fx = cq_t > cq0;
             fx_lo = cq0;
@@ -606,6 +627,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                 ok = search(std::true_type{});
                 if (!(ok = sync(PH_EVICT) && ok)) break;
                 ehi = vload64(&C->stail[1]);
+                fx_long = vload64(&C->hub_created);
             } else {
                 while (ehi > elo) {
                     if (ehi - elo > (unsigned long long)P.big_wave ||
@@ -614,7 +636,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
                         break;
                     }
                     waves++;
-                    for_each_vertex<MODE>(g, P, &C->pc[2], P.EQ, qm, elo, ehi, [&](int v, auto grp) {
+                    for_each_vertex(g, &C->pc[2], P.EQ, qm, elo, ehi, [&](int v, auto grp) {
                         evict_delete_vertex<decltype(grp)>(g, C, P, v, load_vinfo(g, v), e, ls);
                     });
                     if (!(ok = sync(PH_EVICT))) break;
@@ -628,7 +650,6 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
             fx_lo = eq0;
             fx_hi = eq_t;
         }
-        fx_e = e;
         // ------------------------------------------------ next iteration, or hand over
         const unsigned long long nsel = nrem - nrem_next;
         // (a grid-wide insertion logs no evictions: they are about as many as the visits)
@@ -658,8 +679,7 @@ __global__ void __launch_bounds__(MODE == 0 ? kGridThreads : kBlockThreads, MODE
         }
     }
     if (ok && fx) {
-        for_each_vertex<MODE>(g, P, &C->pc[2], FXQ, qm, fx_lo, fx_hi, fixup_body);
-        ok = sync(PH_FIXUP);
+        ok = fixup() && sync(PH_FIXUP);
     }
     // statistics: one atomic per warp
     uint32_t tot[7] = {ls.vis, ls.visl, ls.ev, ls.evl, ls.ch, ls.chl, ls.sel};

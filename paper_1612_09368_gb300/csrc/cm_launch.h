@@ -42,7 +42,7 @@ struct MaintainParams {
     unsigned long long arena_quads;
     uint32_t slab_quads;      // arena quads a warp takes at a time
     int32_t hub_len;          // grid mode: vertices with at least this many slots are scanned grid-wide
-    int32_t block_len;        // vertices with at least this many slots are scanned by a whole block
+    int32_t block_len;        // grid mode, SD fix-up: slots of a long list's chunks
     int32_t claim_max;        // grid-mode task queue: multiple of its fair share of the backlog a warp claims
     int32_t sel_key;          // selection order: 0 fmix64 of the canonical key, 1 the key itself
     int32_t sel_rounds;       // claim rounds per iteration (0 = until the set is maximal)

@@ -94,13 +94,9 @@ enum { N_VIS = 0, N_VISL, N_EV, N_EVL, N_CH, N_CHL, N_SEL };
 __device__ __forceinline__ void note(WarpBuf& B, int what, uint32_t n) {   // one lane of the warp
     B.st[what] += n;
 }
-__device__ __forceinline__ void flush_stats(WarpBuf& B, LocalStats& ls) {
-    const uint32_t mine[7] = {ls.vis, ls.visl, ls.ev, ls.evl, ls.ch, ls.chl, ls.sel};
-#pragma unroll
-    for (int i = 0; i < 7; i++) {
-        const uint32_t t = __reduce_add_sync(0xffffffffu, mine[i]);
-        if (lane_id() == 0) B.st[i] += t;
-    }
+__device__ __forceinline__ void flush_stats(WarpBuf& B, LocalStats& ls) {   // outside searches and fix-ups: selections
+    const uint32_t t = __reduce_add_sync(0xffffffffu, ls.sel);
+    if (lane_id() == 0) note(B, N_SEL, t);
     ls = LocalStats{};
     __syncwarp();
 }
@@ -297,6 +293,78 @@ __device__ __forceinline__ int scan_window(const DevGraph& g, const int32_t* lis
     ne = tot >> 16;
     __syncwarp();
     return tot & 0xFFFF;
+}
+
+// ---------------------------------------------------------------- short lists together
+// Quads [gbase, gend) (at most 128) of the lanes' lists laid end to end: a
+// lane's list is at g.adj + off, has len slots and level k; nq is its number
+// of quads and incl the running sum of those over the lanes.  The candidates
+// go to the front of the buffer, with their owner's lane beside them, and
+// the owners' shares (`part` of scan_window, by KIND) to B.csd.  Returns the
+// number of candidates.  Warp-collective.
+template <int KIND>
+__device__ __forceinline__ int walk_short(const DevGraph& g, WarpBuf& B, long long off, int len, int k, int nq,
+                                          int incl, int gbase, int gend) {
+    const int lane = lane_id();
+    int id[16];
+    uint32_t key[16];
+    unsigned owners = 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const int q = gbase + u * 32 + lane;
+        int o = 0;   // the owner: the first lane whose running quad count exceeds q
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, o + step - 1) <= q) o += step;
+        const long long ob = __shfl_sync(0xffffffffu, off, o);
+        const int ol = __shfl_sync(0xffffffffu, len, o);
+        const int t0 = (q - __shfl_sync(0xffffffffu, incl - nq, o)) * 4;
+        owners |= (unsigned)o << (8 * u);
+        int4 a = make_int4(HOLE, HOLE, HOLE, HOLE);
+        if (q < gend) a = __ldcs(reinterpret_cast<const int4*>(g.adj + ob + t0));
+        id[4 * u] = a.x;
+        id[4 * u + 1] = t0 + 1 < ol ? a.y : HOLE;
+        id[4 * u + 2] = t0 + 2 < ol ? a.z : HOLE;
+        id[4 * u + 3] = t0 + 3 < ol ? a.w : HOLE;
+    }
+#pragma unroll
+    for (int i = 0; i < 16; i++) key[i] = id[i] >= 0 ? g.kc[id[i]] : KEY_DEAD;
+    unsigned mask = 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const int o = (int)((owners >> (8 * u)) & 31u);
+        const int kk = __shfl_sync(0xffffffffu, k, o);
+        int part = 0;
+#pragma unroll
+        for (int i = 4 * u; i < 4 * u + 4; i++) {
+            if (KIND == S_INSERT) {
+                part += (int)key[i] >= 2 * kk + 1;
+                mask |= key[i] == (uint32_t)(2 * kk + 1) ? 1u << i : 0u;
+            } else {
+                if (KIND != S_DELETE) part += key_core(key[i]) >= (KIND == S_ROSE ? kk : kk - 1);
+                mask |= key_core(key[i]) == kk ? 1u << i : 0u;
+            }
+        }
+        if (KIND != S_DELETE && part) atomicAdd(&B.csd[o], part);
+    }
+    const int cnt = __popc(mask);
+    int cinc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, cinc, o);
+        if (lane >= o) cinc += x;
+    }
+    const int nc = __shfl_sync(0xffffffffu, cinc, 31);
+    int at = cinc - cnt;
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        if ((mask >> i) & 1u) {
+            B.id[at] = id[i];
+            B.own[at++] = (uint8_t)((owners >> (8 * (i >> 2))) & 31u);
+        }
+    }
+    __syncwarp();
+    return nc;
 }
 
 // ---------------------------------------------------------------- candidates
@@ -935,63 +1003,7 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
         const int gend = __shfl_sync(0xffffffffu, incl, 31 - __clz(gm));
         B.csd[lane] = 0;
         __syncwarp();
-        int id[16];
-        uint32_t key[16];
-        unsigned owners = 0;
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int q = gbase + u * 32 + lane;
-            int o = 0;   // the owner: the first lane whose running quad count exceeds q
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1)
-                if (__shfl_sync(0xffffffffu, incl, o + step - 1) <= q) o += step;
-            const long long ob = __shfl_sync(0xffffffffu, off, o);
-            const int ol = __shfl_sync(0xffffffffu, len, o);
-            const int t0 = (q - __shfl_sync(0xffffffffu, incl - nq, o)) * 4;
-            owners |= (unsigned)o << (8 * u);
-            int4 a = make_int4(HOLE, HOLE, HOLE, HOLE);
-            if (q < gend) a = __ldcs(reinterpret_cast<const int4*>(g.adj + ob + t0));
-            id[4 * u] = a.x;
-            id[4 * u + 1] = t0 + 1 < ol ? a.y : HOLE;
-            id[4 * u + 2] = t0 + 2 < ol ? a.z : HOLE;
-            id[4 * u + 3] = t0 + 3 < ol ? a.w : HOLE;
-        }
-#pragma unroll
-        for (int i = 0; i < 16; i++) key[i] = id[i] >= 0 ? g.kc[id[i]] : KEY_DEAD;
-        unsigned mask = 0;
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int o = (int)((owners >> (8 * u)) & 31u);
-            const int kk = __shfl_sync(0xffffffffu, k, o);
-            int part = 0;
-#pragma unroll
-            for (int i = 4 * u; i < 4 * u + 4; i++) {
-                if (DEL) {
-                    mask |= key_core(key[i]) == kk ? 1u << i : 0u;
-                } else {
-                    part += (int)key[i] >= 2 * kk + 1;
-                    mask |= key[i] == (uint32_t)(2 * kk + 1) ? 1u << i : 0u;
-                }
-            }
-            if (!DEL && part) atomicAdd(&B.csd[o], part);
-        }
-        const int cnt = __popc(mask);
-        int cinc = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, cinc, o);
-            if (lane >= o) cinc += x;
-        }
-        const int nc = __shfl_sync(0xffffffffu, cinc, 31);
-        int at = cinc - cnt;
-#pragma unroll
-        for (int i = 0; i < 16; i++) {
-            if ((mask >> i) & 1u) {
-                B.id[at] = id[i];
-                B.own[at++] = (uint8_t)((owners >> (8 * (i >> 2))) & 31u);
-            }
-        }
-        __syncwarp();
+        const int nc = walk_short<DEL ? S_DELETE : S_INSERT>(g, B, off, len, k, nq, incl, gbase, gend);
         if (DEL) {
             act_delete<true>(g, C, P, B, W, nc, k, e);
             if (in) {
@@ -1161,57 +1173,184 @@ __device__ __forceinline__ void seed_tasks(Ctl* C, const MaintainParams& P, cons
 }
 
 // ---------------------------------------------------------------- SD fix-up
-// Grid mode's fixup_vertex (cm_vertex.cuh): the SD of a vertex whose core
-// moved in iteration fe, and that of its unmoved neighbours that count it
-// differently now.  Windows of 512 slots as in the search; a group of many
-// warps deals them round robin.  link: iterations follow, so a neighbour at
-// the riser's new level takes it into its record.
-template <int OP, class Grp>
-__device__ __forceinline__ void fixup_wide(const DevGraph& g, const MaintainParams& P, WarpBuf& B, int v, uint32_t fe,
-                                           uint32_t e0, bool link) {
+// Grid mode's fixup_vertex (cm_vertex.cuh), of the vertices whose core moved
+// in iteration fe: their SD, and that of their unmoved neighbours that count
+// them differently now (kk: the neighbours' core).  Like a search step it is
+// a chain of trips (list, keys, change stamps, SD atomics), so what counts is
+// slots in flight and an even share for every warp: long lists in chunks,
+// short ones together.  Measured (GB300) against a warp per list and a block
+// per list of 4096 slots and more: claim phases, where the fix-ups run, of
+// R-MAT scale 24 with 10^6 degree-proportional edges 12.1 -> 8.6 ms (insert)
+// and 10.2 -> 6.6 ms (delete); captured step of 64 Barabasi-Albert graphs
+// 41.6 -> 38.7 ms.  Few moved vertices gain nothing (Erdos-Renyi 10^4
+// vertices, 10^3 edges: 1.06 -> 1.08 ms for four calls).
+//
+// The nc buffered neighbours: of the moved vertex v, or (MANY) of that of
+// lane B.own[i].  link: iterations follow, so a neighbour at a riser's new
+// level takes it into its record.  Warp-collective.
+template <int OP, bool MANY>
+__device__ __forceinline__ void fixup_near(const DevGraph& g, const MaintainParams& P, WarpBuf& B, int nc, int v,
+                                           int kk, uint32_t fe, uint32_t e0, bool link) {
     const int lane = lane_id();
-    const int kn = g.hc[v].x;
-    const int32_t* list = g.adj + g.off[v];
-    const int len = g.end[v];
-    const int kk = OP == 0 ? kn : kn + 1;   // neighbours whose SD counts v differently now
-    int sd = 0, ne = 0;
-    for (int s = Grp::first() * 16; s < len; s += Grp::G * 16) {
-        const int nc = scan_window<OP == 0 ? S_ROSE : S_DROPPED>(g, list, false, s, len, kk, false, B, sd, ne);
-        for (int b0 = 0; b0 < nc; b0 += 128) {
-            int id[4];
-            uint32_t ch[4];
+    for (int b0 = 0; b0 < nc; b0 += 128) {
+        int id[4], ow[4];
+        uint32_t ch[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int i = b0 + j * 32 + lane;
-                id[j] = i < nc ? B.id[i] : -1;
-                ch[j] = i < nc ? __ldcg(g.chg + id[j]) : fe;
-            }
-            // all of this phase's changes to a neighbour go the same way, so
-            // only the update that crosses its core moves its key bit
-            int old[4];
+        for (int j = 0; j < 4; j++) {
+            const int i = b0 + j * 32 + lane;
+            id[j] = i < nc ? B.id[i] : -1;
+            ow[j] = MANY && i < nc ? B.own[i] : 0;
+            ch[j] = i < nc ? __ldcg(g.chg + id[j]) : fe;
+        }
+        // all of this phase's changes to a neighbour go the same way, so
+        // only the update that crosses its core moves its key bit
+        int old[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++)
-                old[j] = ch[j] != fe ? atomicAdd(&g.hc[id[j]].y, OP == 0 ? 1 : -1) : -1;
+        for (int j = 0; j < 4; j++)
+            old[j] = ch[j] != fe ? atomicAdd(&g.hc[id[j]].y, OP == 0 ? 1 : -1) : -1;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                if (ch[j] == fe) continue;
-                if (OP == 0) {
-                    if (old[j] == kk) atomicOr(&g.kc[id[j]], 1u);
-                    if (link) rec_link(P, e0, id[j], kk, v, false);
-                } else if (old[j] == kk + 1) {
-                    atomicAnd(&g.kc[id[j]], ~1u);
-                }
+        for (int j = 0; j < 4; j++) {
+            const int xk = MANY ? __shfl_sync(0xffffffffu, kk, ow[j]) : kk;
+            const int xv = MANY && OP == 0 ? __shfl_sync(0xffffffffu, v, ow[j]) : v;
+            if (ch[j] == fe) continue;
+            if (OP == 0) {
+                if (old[j] == xk) atomicOr(&g.kc[id[j]], 1u);
+                if (link) rec_link(P, e0, id[j], xk, xv, false);
+            } else if (old[j] == xk + 1) {
+                atomicAnd(&g.kc[id[j]], ~1u);
             }
         }
-        __syncwarp();
     }
-    sd = Grp::sum(sd);
-    if (Grp::rank0()) {
-        g.hc[v].y = sd;
-        g.kc[v] = key_of(kn, sd);
-        note(B, N_CH, 1);
-        note(B, N_CHL, len);
+    __syncwarp();
+}
+
+// Lists of more than kShort slots are queued in chunks that any warps take
+// (the task ring is empty between searches; an entry is chunk << 32 | v).
+// The vertex's per-iteration word, which nobody needs before its next
+// iteration, collects its chunks' shares (low half) and arrivals (high half).
+// With a block per list of 4096 slots and more, 40% of the warps' time went
+// to the blocks' barriers and to waiting for the block that drew the longest
+// lists (R-MAT scale 24, 10^6 degree-proportional edges: 1.5*10^9 slots, two
+// thirds of them in 77,000 lists).  Chunks of 1024, 2048 or 4096 slots differ
+// by less than 1%.
+__device__ __forceinline__ int fix_chunk(const MaintainParams& P) { return max(P.block_len & ~(kWindow - 1), kWindow); }
+__device__ __forceinline__ void list_long(const DevGraph& g, Ctl* C, const MaintainParams& P, int v, int len) {
+    if (len <= kShort) return;
+    const int n = (len - 1) / fix_chunk(P) + 1;
+    *iter_word(g, v) = 0;
+    const unsigned long long at = atomicAdd(&C->pc[2], (unsigned long long)n);
+    for (int i = 0; i < n; i++) P.TQ[(at + i) & P.tqmask] = (unsigned long long)i << 32 | (unsigned)v;
+}
+
+// The fix-up of the moved vertices log[lo, hi).  queued: their long lists are
+// nlong queued chunks, which come first; then the vertices, several to a warp
+// when there are more of them than warps, their short lists walked together.
+// Otherwise a warp walks any list.  A warp's first item is dealt by its
+// index, the rest are fetched (C->pc[2], zeroed at every barrier).  Every
+// warp of the launch must call it.
+template <int OP>
+__device__ __forceinline__ void fixup_grid(const DevGraph& g, Ctl* C, const MaintainParams& P, const int32_t* log,
+                                           unsigned long long lo, unsigned long long hi, bool queued,
+                                           unsigned long long nlong, uint32_t fe, uint32_t e0, bool link) {
+    WarpBuf& B = reinterpret_cast<WarpBuf*>(s_search)[threadIdx.x >> 5];
+    const int lane = lane_id();
+    constexpr int up = OP == 0 ? 0 : 1;   // from the moved vertex's core to the neighbours'
+    const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+    const unsigned long long cnt = hi - lo;
+    unsigned many = 1;   // vertices an item
+    unsigned long long all = nlong + cnt;
+    if (queued && cnt > nw) {
+        many = min(((unsigned)cnt - 1) / (unsigned)nw + 1, 32u);
+        all = nlong + ((unsigned)cnt - 1) / many + 1;
     }
+    unsigned long long j = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    while (j < all) {
+        const bool chunk = j < nlong;
+        if (chunk || many == 1) {
+            int v, s0 = 0;
+            if (chunk) {
+                const unsigned long long t = __ldcg(&P.TQ[j & P.tqmask]);
+                v = (int)(uint32_t)t;
+                s0 = (int)(t >> 32) * fix_chunk(P);
+            } else {
+                v = __ldcg(log + ((lo + (j - nlong)) & P.qmask));
+            }
+            const int len = g.end[v], kn = g.hc[v].x;
+            const int32_t* list = g.adj + g.off[v];
+            if (chunk || !queued || len <= kShort) {
+                const int s1 = chunk ? min(s0 + fix_chunk(P), len) : len;
+                int sd = 0, ne = 0;
+                for (int s = s0; s < s1; s += kWindow) {
+                    const int nc = scan_window<OP == 0 ? S_ROSE : S_DROPPED>(g, list, false, s, s1, kn + up, false, B,
+                                                                            sd, ne);
+                    fixup_near<OP, false>(g, P, B, nc, v, kn + up, fe, e0, link);
+                }
+                sd = __reduce_add_sync(0xffffffffu, sd);
+                if (lane == 0) {
+                    bool last = true;
+                    if (chunk) vstore64(&P.TQ[j & P.tqmask], TASK_EMPTY);
+                    if (s1 - s0 < len) {
+                        const unsigned long long o = atomicAdd(iter_word(g, v), 1ull << 32 | (unsigned)sd);
+                        sd += (int)(uint32_t)o;
+                        last = (int)(o >> 32) == (len - 1) / fix_chunk(P);
+                        if (last) *iter_word(g, v) = 0;   // the stamp of no iteration
+                    }
+                    if (last) {
+                        g.hc[v].y = sd;
+                        g.kc[v] = key_of(kn, sd);
+                        note(B, N_CH, 1);
+                        note(B, N_CHL, len);
+                    }
+                }
+            }
+        } else {
+            const unsigned long long i = (j - nlong) * many + lane;
+            bool mine = lane < (int)many && i < cnt;
+            int v = 0, kn = 0, len = 0;
+            long long off = 0;
+            if (mine) {
+                v = __ldcg(log + ((lo + i) & P.qmask));
+                kn = g.hc[v].x;
+                off = g.off[v];
+                len = g.end[v];
+                mine = len <= kShort;   // the others are queued
+            }
+            const int nq = mine ? (len + 3) >> 2 : 0;
+            int incl = nq;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
+            }
+            int gbase = 0;
+            for (unsigned rest = __ballot_sync(0xffffffffu, mine); rest;) {
+                const bool in = ((rest >> lane) & 1u) && incl - gbase <= 128;   // at least one: a list has <= 64 quads
+                const unsigned gm = __ballot_sync(0xffffffffu, in);
+                const int gend = __shfl_sync(0xffffffffu, incl, 31 - __clz(gm));
+                B.csd[lane] = 0;
+                __syncwarp();
+                const int nc = walk_short<OP == 0 ? S_ROSE : S_DROPPED>(g, B, off, len, kn + up, nq, incl, gbase,
+                                                                       gend);
+                if (in) {
+                    const int sd = B.csd[lane];
+                    g.hc[v].y = sd;
+                    g.kc[v] = key_of(kn, sd);
+                }
+                const uint32_t sl = __reduce_add_sync(0xffffffffu, in ? (unsigned)len : 0u);
+                if (lane == 0) {
+                    note(B, N_CH, (uint32_t)__popc(gm));
+                    note(B, N_CHL, sl);
+                }
+                fixup_near<OP, true>(g, P, B, nc, v, kn + up, fe, e0, link);
+                rest &= ~gm;
+                gbase = gend;
+            }
+        }
+        if (all <= nw) break;   // every item was dealt by index
+        if (lane == 0) j = nw + atomicAdd(&C->pc[2], 1ull);
+        j = __shfl_sync(0xffffffffu, j, 0);
+    }
+    __syncwarp();
 }
 
 }  // namespace cm
