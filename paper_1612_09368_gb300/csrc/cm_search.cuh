@@ -37,9 +37,9 @@
 //
 // Measured search time (GB300, one warp per vertex and 128-slot steps -> this
 // layout): Erdos-Renyi, 2*10^6 vertices of degree 8, 10^4 uniform inserts 6.5
-// -> 1.9 ms; 64 Barabasi-Albert graphs (57 iterations) 27 -> 13 ms; R-MAT
+// -> 1.5 ms; 64 Barabasi-Albert graphs (57 iterations) 27 -> 11 ms; R-MAT
 // scale 24, 10^3 degree-proportional inserts (4*10^5 vertices visited,
-// 3.8*10^8 slots) 7.5 -> 5.0 ms, of which the key gathers alone are 1.3 ms
+// 3.8*10^8 slots) 7.5 -> 4.1 ms, of which the key gathers alone are 1.3 ms
 // at the 300 G gathers/s (one lane per clock and SM) that a kernel doing
 // nothing else reaches.
 //
