@@ -448,8 +448,8 @@ __device__ __forceinline__ void act_insert(const DevGraph& g, Ctl* C, const Main
 }
 
 // The recorded ids [i0, i1) of an evicted vertex at level k.  Its expansion
-// in this iteration visited the candidates among them, so their words carry
-// the iteration's stamp and a plain add does.  all: the record is of an
+// in this iteration has visited the candidates among them (run_batch sees to
+// that), so their words carry the iteration's stamp and a plain add does.  all: the record is of an
 // earlier iteration and its marks are out of date (ids have risen above k,
 // SDs have grown), so the keys tell who is a candidate now.  Warp-collective.
 __device__ __forceinline__ void act_recorded(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
@@ -929,9 +929,16 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
     int4 hdr = make_int4(0, 0, 0, -1);
     if (!DEL && vert && len > kShort && rec_stamp(rec) >= e0)
         hdr = __ldcg(reinterpret_cast<const int4*>(P.arena + 4 * (rec >> 30)));
-    // whose record will do: at its level k, or made in this very iteration
+    // Whose record will do.  For a frontier vertex: one at its level k.  For an
+    // evicted one: one made in this very iteration, which is published after
+    // the walk that visited its candidates, or an earlier one at its level if
+    // the vertex expanded early: the processed flag, without which nobody
+    // evicts it, came after its visits then.  In the paper's order the flag
+    // comes first, so an eviction can overtake the visits and meet words that
+    // are still of older iterations, which act_recorded must not: the list.
     const bool now = rec_stamp(rec) == e;
-    const unsigned use = __ballot_sync(0xffffffffu, hdr.x <= hdr.y && hdr.y > 0 && (hdr.w == k || (now && !front)));
+    const bool fits = front ? hdr.w == k : now || (hdr.w == k && expand_early(P));
+    const unsigned use = __ballot_sync(0xffffffffu, hdr.x <= hdr.y && hdr.y > 0 && fits);
     // lists of more than kShort slots, one after another
     for (unsigned m = __ballot_sync(0xffffffffu, vert && len > kShort); m; m &= m - 1) {
         const int src = __ffs(m) - 1;
