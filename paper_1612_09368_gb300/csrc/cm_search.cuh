@@ -485,11 +485,14 @@ __device__ __forceinline__ void act_recorded(const DevGraph& g, Ctl* C, const Ma
 }
 
 // Core-k neighbours id[] (-1: none) of vertices evicted by a deletion, with
-// their words, thresholds SD - k + 1 and change stamps as read.
+// their words, thresholds SD - k + 1 and change stamps as read; low[]: the low
+// half of a current word counted at their level.  One that has left meanwhile
+// and passes for level k (level_bits) may be counted once more, which does no
+// harm, but not evicted again.
 template <int J>
 __device__ __forceinline__ void delete_words(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
-                                             const int (&id)[J], const int (&thr)[J], const unsigned long long (&s)[J],
-                                             const uint32_t (&ch)[J], uint32_t e) {
+                                             const int (&id)[J], const int (&thr)[J], const uint32_t (&low)[J],
+                                             const unsigned long long (&s)[J], const uint32_t (&ch)[J], uint32_t e) {
     const unsigned long long inc = 1ull << 32;
     unsigned long long r[J];
     unsigned go = 0;
@@ -499,21 +502,21 @@ __device__ __forceinline__ void delete_words(const DevGraph& g, Ctl* C, const Ma
         const bool same = same_iter(wz(s[j]), e);
         if (id[j] < 0 || ch[j] == e || thr[j] <= 0 || (same && ww(s[j]) >= thr[j])) continue;
         go |= 1u << j;
-        r[j] = same ? atomicAdd(iter_word(g, id[j]), inc)
-                    : atomicCAS(iter_word(g, id[j]), s[j], inc | (unsigned long long)(e << 2));
+        r[j] = same ? atomicAdd(iter_word(g, id[j]), inc) : atomicCAS(iter_word(g, id[j]), s[j], inc | low[j]);
     }
     unsigned em = 0;
 #pragma unroll
     for (int j = 0; j < J; j++) {
         if (!((go >> j) & 1u)) continue;
-        int oc = 0;
-        if (same_iter(wz(s[j]), e)) {
-            oc = ww(r[j]);
-        } else if (r[j] != s[j]) {   // someone touched it first: restamp if needed, then add
-            make_current(g, C, id[j], e, r[j]);
-            oc = ww(atomicAdd(iter_word(g, id[j]), inc));
+        if (!same_iter(wz(s[j]), e)) {
+            if (r[j] == s[j]) {   // first to touch it in this iteration
+                r[j] = low[j];
+            } else {              // someone did it first: restamp if needed, then add
+                make_current(g, C, id[j], e, r[j], low[j] & 3u);
+                r[j] = atomicAdd(iter_word(g, id[j]), inc);
+            }
         }
-        if (oc + 1 == thr[j]) {
+        if (wz(r[j]) == low[j] && ww(r[j]) + 1 == thr[j]) {
             g.chg[id[j]] = e;
             em |= 1u << j;
         }
@@ -525,7 +528,7 @@ __device__ __forceinline__ void delete_words(const DevGraph& g, Ctl* C, const Ma
 // deletion: each loses one support, initially its SD, and leaves when its
 // count of evicted neighbours reaches SD - k + 1 (Algorithm 7).  Evicted
 // vertices (chg == e) are skipped: their cores already dropped, so one that
-// fell from k + 1 would pass for level k.
+// fell from k + 1 would pass for level k (one that is missed: see level_bits).
 template <bool MANY, int J = 4>
 __device__ __forceinline__ void act_delete(const DevGraph& g, Ctl* C, const MaintainParams& P, WarpBuf& B, Walker& W,
                                            int nc, int k, uint32_t e) {
@@ -533,7 +536,7 @@ __device__ __forceinline__ void act_delete(const DevGraph& g, Ctl* C, const Main
     for (int b0 = 0; b0 < nc; b0 += 32 * J) {
         int id[J], thr[J];
         unsigned long long s[J];
-        uint32_t ch[J];
+        uint32_t ch[J], low[J];
 #pragma unroll
         for (int j = 0; j < J; j++) {
             const int i = b0 + j * 32 + lane;
@@ -541,10 +544,11 @@ __device__ __forceinline__ void act_delete(const DevGraph& g, Ctl* C, const Main
             const int o = MANY && i < nc ? B.own[i] : 0;
             const int kk = MANY ? __shfl_sync(0xffffffffu, k, o) : k;
             s[j] = id[j] >= 0 ? __ldcg(iter_word(g, id[j])) : 0ull;
-            ch[j] = id[j] >= 0 ? __ldcg(g.chg + id[j]) : e;   // from L2: never older than the key
+            ch[j] = id[j] >= 0 ? __ldcg(g.chg + id[j]) : e;
             thr[j] = id[j] >= 0 ? g.hc[id[j]].y - kk + 1 : 0;
+            low[j] = e << 2 | level_bits(kk);
         }
-        delete_words<J>(g, C, P, B, W, id, thr, s, ch, e);
+        delete_words<J>(g, C, P, B, W, id, thr, low, s, ch, e);
     }
 }
 
@@ -871,7 +875,8 @@ __device__ __forceinline__ void lone_tiny(const DevGraph& g, Ctl* C, const Maint
         const uint32_t ch[1] = {x >= 0 ? __ldcg(g.chg + x) : e};
         const int thr[1] = {x >= 0 ? g.hc[x].y - k + 1 : 0};
         const int id[1] = {key_core(key) == k ? x : -1};
-        delete_words<1>(g, C, P, B, W, id, thr, s, ch, e);
+        const uint32_t low[1] = {e << 2 | level_bits(k)};
+        delete_words<1>(g, C, P, B, W, id, thr, low, s, ch, e);
         if (lane == 0) {
             g.hc[v].x = k - 1;
             g.kc[v] = key_of(k - 1, 0);   // bit set by the SD fix-up
@@ -1138,11 +1143,14 @@ __device__ __forceinline__ bool async_search(const DevGraph& g, Ctl* C, const Ma
             held &= ~got;
             ndone += (unsigned)__popc(got);
         }
-        // The poll acquires what the producers of its tasks wrote.  Beyond that
-        // nothing here may be older than a task: words, change stamps and
-        // records are read at L2 or with acquire, and the keys may lag (a core
-        // that has dropped meanwhile is recognised by its change stamp).  Only a
-        // chunk task needs more than its own producer's writes, its hub item.
+        // Tasks are stored without a release, so a poll orders nothing but the
+        // task.  A vertex task needs no more: what it reads of its vertex is
+        // fixed since the last barrier, counts and flags are changed by atomics
+        // whose results their callers had before they stored a task, a record's
+        // word is published behind a fence and read with acquire, and keys and
+        // change stamps may lag (see level_bits; an insertion changes neither
+        // during its search).  A chunk task needs its hub item, which is
+        // written before a fence that this one meets.
         __syncwarp();
         if (__any_sync(0xffffffffu, t != TASK_EMPTY && (int)(t >> 62) == T_CHUNK)) __threadfence();
         run_batch<DEL>(g, C, P, B, W, e, e0, t);

@@ -15,8 +15,9 @@
 // with an older stamp reads as "no flags, count 0"; the first update in an
 // iteration stamps it with one CAS, later updates are single atomicAdd /
 // atomicOr operations on the 64-bit word.  Insert flags: 1 visited (in a
-// frontier), 2 processed (CSD added); w = support.  Delete: w = evicted
-// neighbours.
+// frontier), 2 processed (CSD added); w = support.  Delete flags: the low two
+// bits of the level that the vertex is counted at (see level_bits); w =
+// evicted neighbours.
 #pragma once
 #include "cm_common.cuh"
 #include "cm_launch.h"
@@ -41,16 +42,26 @@ __device__ __forceinline__ unsigned long long* iter_word(const DevGraph& g, int 
 __device__ __forceinline__ uint32_t wz(unsigned long long x) { return (uint32_t)x; }
 __device__ __forceinline__ int32_t ww(unsigned long long x) { return (int32_t)(uint32_t)(x >> 32); }
 
-// Stamps v's word with iteration e if it is older (count 0, no flags).
-// `seen` is a value of the word the caller already read (from the 16-byte
-// vertex gather), which saves a load: a word stamped e stays stamped e for
-// the rest of the iteration.  Retries are bounded; past the bound an error
-// is recorded.
-__device__ __forceinline__ void make_current(const DevGraph& g, Ctl* C, int v, uint32_t e, unsigned long long seen) {
+// Deletion: the flags of a word counted at level k.  In grid mode a vertex's
+// key, change stamp and word are read with nothing to order them, so one that
+// has just left level k + 1 may pass for one of level k: its key read new, its
+// stamp old.  Its count then stands at SD - k, one below the threshold of level
+// k, and a second eviction would lower its core by two.  Whoever reaches a
+// threshold therefore compares the word's level as well, which came with the
+// first update of the iteration: it is part of what its atomic returns.  (A
+// root has no updates, but its change stamp was set before the last barrier.)
+__device__ __forceinline__ uint32_t level_bits(int k) { return (uint32_t)k & 3u; }
+
+// Stamps v's word with iteration e if it is older (count 0, the given flags).
+// `seen` is a value of the word the caller already read, which saves a load: a
+// word stamped e stays stamped e for the rest of the iteration.  Retries are
+// bounded; past the bound an error is recorded.
+__device__ __forceinline__ void make_current(const DevGraph& g, Ctl* C, int v, uint32_t e, unsigned long long seen,
+                                             uint32_t flags = 0u) {
     if (same_iter(wz(seen), e)) return;
     unsigned long long* p = iter_word(g, v);
     unsigned long long old = seen;
-    const unsigned long long fresh = (unsigned long long)(e << 2);
+    const unsigned long long fresh = (unsigned long long)((e << 2) | flags);
     for (int tries = 0; tries < (1 << 20); tries++) {
         if (same_iter(wz(old), e)) return;
         unsigned long long prev = atomicCAS(p, old, fresh);
@@ -115,12 +126,13 @@ __device__ __forceinline__ bool visit(const DevGraph& g, Ctl* C, int v, uint32_t
 // The same two operations for the four slots of a lane's scan step, with
 // the four first atomics issued before any result is used; a slot whose
 // word changed since it was gathered takes the slow path of add_word /
-// visit.  Slots with want[q] / cand[q] false are left alone.
+// visit.  Slots with want[q] / cand[q] false are left alone.  flags: those of
+// a word that add_word4 stamps (a deletion's level).
 __device__ __forceinline__ void add_word4(const DevGraph& g, Ctl* C, const int (&v)[4], const bool (&want)[4],
                                           uint32_t e, int32_t delta, const unsigned long long (&seen)[4],
-                                          uint32_t (&oflags)[4], int32_t (&ocount)[4]) {
+                                          uint32_t (&oflags)[4], int32_t (&ocount)[4], uint32_t flags = 0u) {
     const unsigned long long inc = (unsigned long long)(uint32_t)delta << 32;
-    const unsigned long long fresh = inc | (unsigned long long)(e << 2);
+    const unsigned long long fresh = inc | (unsigned long long)((e << 2) | flags);
     unsigned long long r[4];
 #pragma unroll
     for (int q = 0; q < 4; q++) {
@@ -137,7 +149,7 @@ __device__ __forceinline__ void add_word4(const DevGraph& g, Ctl* C, const int (
             oflags[q] = wz(r[q]) & 3u;
             ocount[q] = ww(r[q]);
         } else if (r[q] != seen[q]) {   // someone touched it first: restamp if needed, then add
-            make_current(g, C, v[q], e, r[q]);
+            make_current(g, C, v[q], e, r[q], flags);
             const unsigned long long old = atomicAdd(iter_word(g, v[q]), inc);
             oflags[q] = wz(old) & 3u;
             ocount[q] = ww(old);
@@ -459,7 +471,7 @@ __device__ __forceinline__ void evict_del_range(const DevGraph& g, Ctl* C, const
             cand[q] = h[q].x == k && !gone && c[q] != e;
             sw[q] = word_of(h[q]);
         }
-        add_word4(g, C, w, cand, e, 1, sw, of, oc);
+        add_word4(g, C, w, cand, e, 1, sw, of, oc, level_bits(k));
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             p[q] = cand[q] && oc[q] + 1 == h[q].y - k + 1;

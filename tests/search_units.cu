@@ -67,5 +67,52 @@ extern "C" int unit_evict(int n, int len, int2* hc, unsigned long long* hw, uint
     return 0;
 }
 
+// Lane l handles entries l, l + 32, ... of a deletion's core-k neighbours.
+template <int J>
+__global__ void delete_kernel(DevGraph g, Ctl* C, MaintainParams P, const int32_t* id, const int32_t* thr,
+                              const unsigned long long* s, const uint32_t* ch, uint32_t e, int k) {
+    WarpBuf& B = *reinterpret_cast<WarpBuf*>(s_search);
+    Walker W{0, 1, false, 0};
+    int i[J], t[J];
+    unsigned long long w[J];
+    uint32_t c[J], low[J];
+#pragma unroll
+    for (int j = 0; j < J; j++) {
+        const int a = j * 32 + lane_id();
+        i[j] = id[a];
+        t[j] = thr[a];
+        w[j] = s[a];
+        c[j] = ch[a];
+        low[j] = e << 2 | level_bits(k);
+    }
+    delete_words<J>(g, C, P, B, W, i, t, low, w, c, e);
+}
+
+// 32 entries (wide: 128) at level k.  evicted: those logged.
+extern "C" int unit_delete(int wide, int n, unsigned long long* hw, uint32_t* chg, unsigned long long* tq, int tq_size,
+                           int32_t* eq, int ring, Ctl* ctl, const int32_t* id, const int32_t* thr,
+                           const unsigned long long* s, const uint32_t* ch, unsigned e, int k,
+                           unsigned long long* evicted) {
+    DevGraph g{};
+    g.n = n;
+    g.hw = hw;
+    g.chg = chg;
+    MaintainParams P{};
+    P.g = g;
+    P.ctl = ctl;
+    P.EQ = eq;
+    P.qmask = (unsigned long long)ring - 1;
+    P.TQ = tq;
+    P.tqmask = (unsigned long long)tq_size - 1;
+    if (cudaMemset(ctl, 0, sizeof(Ctl)) != cudaSuccess) return 1;
+    if (wide) delete_kernel<4><<<1, 32, kSearchSmem>>>(g, ctl, P, id, thr, s, ch, e, k);
+    else delete_kernel<1><<<1, 32, kSearchSmem>>>(g, ctl, P, id, thr, s, ch, e, k);
+    Ctl h;
+    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return 2;
+    *evicted = h.tail[1];
+    return h.error ? 3 : 0;
+}
+
 extern "C" int unit_ctl_bytes() { return (int)sizeof(Ctl); }
 extern "C" int unit_hub_ring() { return (int)kHubRing; }

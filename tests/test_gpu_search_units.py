@@ -83,3 +83,43 @@ def test_eviction_from_an_earlier_iterations_record(units, length, hub_len, visi
     want[cand] = ((np.uint64(39) << np.uint64(32)) | np.uint64(e << 2 | 3)) if visited else \
         np.uint64(0xFFFFFFFF00000000) | np.uint64(e << 2)
     assert (got == want).all()
+
+
+@pytest.mark.parametrize("wide", [0, 1])
+def test_a_vertex_leaves_once_whatever_stamp_was_read(units, wide):
+    """A deletion's neighbours as read with an old change stamp: one that has
+    left level k + 1 meanwhile (its count is one below the threshold of level k)
+    is not evicted again, the others leave when their count reaches it.  A
+    word carries the low bits of its level."""
+    import torch
+    e, k, m = 9, 5, 128 if wide else 32
+    i = np.arange(m)
+    kind = i % 5            # 0 left meanwhile; 1 leaves now; 2, 4 stay; 3 leaves at the first touch
+    sd = k + 2 + i % 7
+    count = np.where((kind == 2) | (kind == 4), 0, sd - k)
+    sd[kind == 3] = k
+    thr = (sd - k + 1).astype(np.int32)
+    level = np.where(kind == 0, k + 1, k).astype(np.uint64)
+    word = (count.astype(np.uint64) << np.uint64(32)) | np.uint64(e << 2) | (level & np.uint64(3))
+    word[(kind == 3) | (kind == 4)] = np.uint64(77) << np.uint64(32) | np.uint64((e - 1) << 2)
+    read = np.full(m, e - 2, np.uint32)
+    chg = np.where(kind == 0, e, e - 2).astype(np.uint32)
+    d_word, d_chg = _dev(word.view(np.int64)), _dev(chg.view(np.int32))
+    ring, tqs = 1 << 10, 1 << 19
+    tq = torch.full((tqs,), -1, dtype=torch.int64, device="cuda")
+    eq = torch.full((ring,), -1, dtype=torch.int32, device="cuda")
+    ctl = torch.zeros(units.unit_ctl_bytes(), dtype=torch.uint8, device="cuda")
+    args = [_dev(x) for x in (i.astype(np.int32), thr, word.view(np.int64), read.view(np.int32))]
+    out = ctypes.c_uint64()
+    rc = units.unit_delete(wide, m, _p(d_word), _p(d_chg), _p(tq), tqs, _p(eq), ring, _p(ctl), *[_p(x) for x in args], e,
+                           k, ctypes.byref(out))
+    assert rc == 0
+    leave = np.flatnonzero((kind == 1) | (kind == 3))
+    assert out.value == len(leave)
+    assert (np.sort(eq.cpu().numpy()[: len(leave)]) == leave).all()
+    want = chg.copy()
+    want[leave] = e
+    assert (d_chg.cpu().numpy().view(np.uint32) == want).all()
+    got = d_word.cpu().numpy().view(np.uint64)
+    first = np.uint64(1) << np.uint64(32) | np.uint64(e << 2 | k & 3)
+    assert (got == np.where((kind == 3) | (kind == 4), first, word + (np.uint64(1) << np.uint64(32)))).all()
