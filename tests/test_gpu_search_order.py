@@ -74,3 +74,29 @@ def test_lists_around_the_short_limit(cm, d, expand_early):  # noqa: F811
         assert (g.cores() == ref).all(), b
         assert (g.superior_degrees() == _sd(n, cur, ref)).all(), b
     g.close()
+
+
+@pytest.mark.parametrize("leave", [4, 16, 64, 400])
+def test_searches_handed_from_one_block_to_the_grid(cm, leave):  # noqa: F811
+    """Searches that begin in single-block waves and go on grid-wide: both
+    leave the vertices' words as the other expects them."""
+    rng = np.random.default_rng(leave)
+    n = 4000
+    x = rng.integers(0, n, (5 * n, 2))
+    y = x[x[:, 0] != x[:, 1]]
+    keys = np.unique(np.minimum(y[:, 0], y[:, 1]) * n + np.maximum(y[:, 0], y[:, 1]))
+    e = _pairs(n, keys)
+    g = cm.CoreGraph(n, e, block_mode_enter=1 << 30, block_mode_leave=leave)
+    ref = oracle.OracleGraph(n, e, mode=oracle.SUPERIOR)
+    hot = rng.choice(n, 60, replace=False)
+    for b in range(6):
+        new = np.stack([rng.choice(hot, 300), rng.integers(0, n, 300)], 1).astype(np.int32)
+        new = new[new[:, 0] != new[:, 1]]
+        old = np.concatenate([new[::2], e[rng.choice(len(e), 400, replace=False)]]).astype(np.int32)
+        for f, r, batch in ((g.insert_edges, ref.insert_edges, new), (g.delete_edges, ref.delete_edges, old)):
+            assert f(batch) == r(batch)
+            assert g.stats()["iterations"] == ref.last_iterations() > 1
+            assert (g.cores() == ref.cores()).all(), b
+    r = g.check()
+    assert [r[k] for k in ("sd_mismatches", "key_mismatches", "kcore_violations")] == [0] * 3
+    g.close()
