@@ -72,12 +72,16 @@ struct cm_graph {
     HubItem* HQ = nullptr;
     unsigned long long* TQ = nullptr;   // grid-mode task queue (TASK_EMPTY = all ones when free)
     unsigned long long tq_size = 0;
-    // records of the grid-mode search (cm_search.cuh): per vertex
-    // a stamped position in the arena
+    // records of the grid-mode search (cm_search.cuh): a word per vertex and an
+    // arena, in rec_base or, if that is too small, in rec_mem (ensure_records)
     unsigned long long* rec = nullptr;
-    size_t rec_size = 0;
+    size_t rec_n = 0;                    // vertices with a word (0: no records)
     int32_t* arena = nullptr;
     unsigned long long arena_quads = 0;
+    unsigned char* rec_base = nullptr;   // kRecBase bytes, for the handle's life
+    unsigned char* rec_mem = nullptr;
+    size_t rec_bytes = 0;                // of rec_mem
+    size_t rec_refused = 0;              // do not ask for up to this many bytes again
     int32_t hub_len = 1024;
     int32_t block_len = 4096, block_len_del = 1024;
     int32_t claim_max = 1;
@@ -280,11 +284,7 @@ static int ensure_index(cm_graph* h, long long adding) {
 // frontier and being evicted once per iteration, plus the chunk tasks of
 // high-degree lists (three passes per list, at least 128 slots per hub) and
 // the claims warps make past the tail.
-static int ensure_records(cm_graph* h);
-
 static int ensure_tasks(cm_graph* h) {
-    int rc = ensure_records(h);
-    if (rc) return rc;
     const unsigned long long need =
         pow2_at_least(2ull * (unsigned long long)h->ncap + (unsigned long long)h->g.adj_cap / 32 + (1ull << 18));
     if (need <= h->tq_size) return CM_OK;
@@ -300,32 +300,48 @@ static int ensure_tasks(cm_graph* h) {
     return CM_OK;
 }
 
-// Records of the search: a word per vertex, and an arena of two thirds of the
-// adjacency pool's bytes for a launch's records (a search that fills it scans
-// the lists of the vertices left out).
+// Records of the insertion search: a word per vertex, and an arena of two
+// thirds of the adjacency pool's bytes for a launch's records.  They only save
+// time (a search that finds no room, or no records at all, scans the lists
+// again), so memory that cannot be had for them is no error: a smaller arena
+// is tried, then the block that every handle has.  Deletions need none.
+// Nothing in them outlives a launch, so the old memory goes back first.
+// A refused size is not asked for again until a quarter more is wanted.
+constexpr size_t kRecBase = 4ull << 20;
 static int ensure_records(cm_graph* h) {
-    if (h->rec_size < (size_t)h->ncap) {
-        unsigned long long* q = (unsigned long long*)dalloc(h, (size_t)h->ncap * 8);
-        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the search records");
-        CK(h, cudaMemsetAsync(q, 0, (size_t)h->ncap * 8, h->stream));   // stamp 0 names no iteration
-        if (h->rec) {
-            CK(h, cudaStreamSynchronize(h->stream));
-            dfree(h, h->rec, h->rec_size * 8);
-        }
-        h->rec = q;
-        h->rec_size = (size_t)h->ncap;
-    }
     const unsigned long long quads = (unsigned long long)h->g.adj_cap / 6 + 1024;
-    if (h->arena_quads < quads) {
-        int32_t* q = (int32_t*)dalloc(h, (size_t)quads * 16);
-        if (!q) return set_err(h, CM_ERR_OOM, "out of device memory for the record arena");
-        if (h->arena) {
-            CK(h, cudaStreamSynchronize(h->stream));
-            dfree(h, h->arena, (size_t)h->arena_quads * 16);
-        }
-        h->arena = q;
-        h->arena_quads = quads;
+    const size_t words = ((size_t)h->ncap * 8 + 15) & ~(size_t)15, need = words + (size_t)quads * 16;
+    const bool valid = h->rec_n >= (size_t)h->ncap;
+    if (valid && h->arena_quads >= quads) return CM_OK;
+    if (need > kRecBase && need <= h->rec_refused && (valid || h->rec_n == 0)) return CM_OK;
+    if (h->rec_mem) {
+        CK(h, cudaStreamSynchronize(h->stream));
+        dfree(h, h->rec_mem, h->rec_bytes);
+        h->rec_mem = nullptr;
+        h->rec_bytes = 0;
     }
+    unsigned char* at = h->rec_base;
+    size_t bytes = kRecBase, n = (size_t)h->ncap;
+    if (need > kRecBase) {
+        for (int part = 1; part <= 8 && !h->rec_mem; part *= 2) {
+            bytes = words + (size_t)(quads / part) * 16;
+            if (bytes > kRecBase) h->rec_mem = (unsigned char*)dalloc(h, bytes);
+            h->rec_refused = h->rec_mem && part == 1 ? 0 : need + need / 4;
+        }
+        if (h->rec_mem) {
+            at = h->rec_mem;
+            h->rec_bytes = bytes;
+        } else {
+            bytes = kRecBase;
+            if (words > kRecBase / 2) n = 0;   // no records
+        }
+    }
+    const size_t used = n ? words : 16;
+    CK(h, cudaMemsetAsync(at, 0, used, h->stream));   // stamp 0 names no iteration
+    h->rec = (unsigned long long*)at;
+    h->rec_n = n;
+    h->arena = (int32_t*)(at + used);
+    h->arena_quads = n ? (bytes - used) / 16 : 0;
     return CM_OK;
 }
 
@@ -435,8 +451,8 @@ static void free_all(cm_graph* h) {
     dfree(h, h->OVL, qn * 4);
     dfree(h, h->HQ, kHubRing * sizeof(HubItem));
     dfree(h, h->TQ, h->tq_size * 8);
-    dfree(h, h->rec, h->rec_size * 8);
-    dfree(h, h->arena, (size_t)h->arena_quads * 16);
+    dfree(h, h->rec_base, kRecBase);
+    dfree(h, h->rec_mem, h->rec_bytes);
     dfree(h, h->dbatch, (size_t)h->batch_cap * 8);
     dfree(h, h->bset, h->bset_size * sizeof(BSet));
     dfree(h, h->R0, (size_t)h->rcap * sizeof(REdge));
@@ -536,6 +552,8 @@ static int create_common(int32_t n, const int32_t* edges, long long m, const int
     CK(h, cudaMemset(h->ctl, 0, sizeof(Ctl)));
     h->HQ = (HubItem*)dalloc(h, kHubRing * sizeof(HubItem));
     if (!h->HQ) return set_err(h, CM_ERR_OOM, "out of device memory for the hub items");
+    h->rec_base = (unsigned char*)dalloc(h, kRecBase);
+    if (!h->rec_base) return set_err(h, CM_ERR_OOM, "out of device memory for the search records");
     CK(h, cudaMallocHost(&h->hctl, sizeof(Ctl)));
     memset(h->hctl, 0, sizeof(Ctl));
     h->g.slack_pct = h->opt.slack_pct;
@@ -709,7 +727,8 @@ static void add_maintain_counters(cm_stats& s, const unsigned long long* st, con
 
 // Parameters of a maintenance launch pair from the handle: its buffers and
 // the schedule its options set (a captured step overrides the schedule).
-// The task queue must be allocated first (ensure_tasks).
+// The task queue, and for an insertion the records, must be in place first
+// (ensure_tasks, ensure_records).
 static MaintainParams handle_params(const cm_graph* h, int op) {
     MaintainParams p{};
     p.g = h->g;
@@ -734,6 +753,7 @@ static MaintainParams handle_params(const cm_graph* h, int op) {
     p.rec = h->rec;
     p.arena = h->arena;
     p.arena_quads = h->arena_quads;
+    p.rec_mask = h->rec_n ? -1 : 0;
     {   // a slab for every warp of the largest grid takes a quarter of the arena at most
         const unsigned long long per = h->arena_quads / (4ull * (unsigned long long)h->num_sms * 32ull);
         p.slab_quads = (uint32_t)(per < 32 ? 32 : per > 1024 ? 1024 : per);
@@ -772,7 +792,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
         CK(h, cudaMemsetAsync(g.chg, 0, (size_t)h->n * 4, h->stream));
         CK(h, cudaMemsetAsync(g.taken, 0, (size_t)h->n * 4, h->stream));
         CK(h, cudaMemsetAsync(g.hw, 0, (size_t)h->n * sizeof(unsigned long long), h->stream));
-        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, h->stream));
+        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_n * 8, h->stream));
         h->epoch = 1;
     }
     // where the iterations start: all kept edges remain, in R0.  Every call
@@ -850,6 +870,7 @@ static int update_device(cm_graph* h, int op, const int32_t* dE, long long k, in
             return set_err(h, CM_ERR_LIMIT, "structure update failed with device error %d", c.error);
         }
     } else if (nrem0 > 0) {
+        if (op == CM_OP_INSERT && (rc = ensure_records(h))) return rc;
         MaintainParams p = handle_params(h, op);
         p.max_iters = nrem0 + 1;
         int blocks, threads;
@@ -1718,12 +1739,13 @@ static int step_prepare(cm_step* s, long long kins) {
     const long long kmax = s->max_ins > s->max_del ? s->max_ins : s->max_del;
     if ((rc = ensure_batch(h, kmax))) return rc;
     if ((rc = ensure_tasks(h))) return rc;
+    if (s->max_ins > 0 && (rc = ensure_records(h))) return rc;
     if (h->epoch > 0x3F000000u) {   // 30-bit stamps about to wrap: clear them
         DevGraph& g = h->g;
         CK(h, cudaMemsetAsync(g.chg, 0, (size_t)h->n * 4, h->stream));
         CK(h, cudaMemsetAsync(g.taken, 0, (size_t)h->n * 4, h->stream));
         CK(h, cudaMemsetAsync(g.hw, 0, (size_t)h->n * sizeof(unsigned long long), h->stream));
-        CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, h->stream));
+        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_n * 8, h->stream));
         h->epoch = 1;
     }
     *s->hEpoch = h->epoch;
@@ -1911,7 +1933,7 @@ static int snap_copy(cm_graph* h, Snapshot& z, bool save) {
         h->idx_tomb = z.idx_tomb;
         h->epoch = z.epoch;
         h->n = z.n;
-        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_size * 8, st));   // the stamps run again from z.epoch
+        if (h->rec) CK(h, cudaMemsetAsync(h->rec, 0, h->rec_n * 8, st));   // the stamps run again from z.epoch
     }
     return CM_OK;
 }

@@ -41,6 +41,7 @@ struct MaintainParams {
     int32_t* arena;
     unsigned long long arena_quads;
     uint32_t slab_quads;      // arena quads a warp takes at a time
+    int32_t rec_mask;         // -1; 0 if there is no memory for records: every vertex reads rec[0], which names none
     int32_t hub_len;          // grid mode: vertices with at least this many slots are scanned grid-wide
     int32_t block_len;        // grid mode, SD fix-up: slots of a long list's chunks
     int32_t claim_max;        // grid-mode task queue: multiple of its fair share of the backlog a warp claims

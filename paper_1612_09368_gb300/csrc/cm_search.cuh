@@ -123,7 +123,7 @@ __device__ __forceinline__ uint32_t rec_stamp(unsigned long long w) { return (ui
 // above, or appends it.  Runs between searches, when nobody reads records.
 __device__ __forceinline__ void rec_link(const MaintainParams& P, uint32_t e0, int v, int k, int other,
                                          bool other_above) {
-    const unsigned long long w = vload64(&P.rec[v]);
+    const unsigned long long w = vload64(&P.rec[v & P.rec_mask]);
     if (rec_stamp(w) < e0) return;
     int32_t* r = P.arena + 4 * (w >> 30);
     const int room = vload32(&r[1]);
@@ -927,7 +927,7 @@ __device__ __forceinline__ void run_batch(const DevGraph& g, Ctl* C, const Maint
         const int2 c = g.hc[v];
         off = g.off[v];
         len = g.end[v];
-        if (!DEL) rec = ld_acquire64(&P.rec[v]);
+        if (!DEL) rec = ld_acquire64(&P.rec[v & P.rec_mask]);
         k = c.x;
         sd = c.y;
     }

@@ -48,6 +48,7 @@ extern "C" int unit_evict(int n, int len, int2* hc, unsigned long long* hw, uint
     P.TQ = tq;
     P.tqmask = (unsigned long long)tq_size - 1;
     P.rec = rec;
+    P.rec_mask = -1;
     P.arena = arena;
     P.arena_quads = quads;
     P.slab_quads = 32;
