@@ -68,7 +68,8 @@ typedef struct cm_options {
     int32_t slack_pct;      /* per-vertex adjacency headroom in percent (default 25) */
     int32_t min_cap;        /* minimum adjacency slots per vertex, rounded up to 4 (default 4) */
     int32_t block_threads;  /* unused (kept for layout): every persistent kernel has its own block size */
-    int32_t blocks_per_sm;  /* resident blocks per SM of the persistent kernels; 0 = occupancy limit */
+    int32_t blocks_per_sm;  /* resident blocks per SM of the grid-wide maintenance kernels; 0 = occupancy limit
+                               (the peel always takes one block per SM) */
     int32_t max_sms;        /* SMs the persistent kernels may fill; 0 = all (lower it to share the GPU) */
     int32_t block_mode_edges; /* single-block mode only while at most this many edges remain (16384;
                                  negative = never leave grid mode) */
@@ -134,9 +135,9 @@ typedef struct cm_stats {
     int64_t selected;        /* edges selected, summed over iterations (= applied) */
     int64_t remaining_sum;   /* remaining edges at iteration start, summed */
     int64_t visited;         /* vertices entered into the candidate set (insert) */
-    int64_t visited_slots;   /* adjacency slots of those vertices */
+    int64_t visited_slots;   /* slots read for them: adjacency slots, or the ids of a vertex walked from its record */
     int64_t evicted;         /* vertices evicted by support waves */
-    int64_t evicted_slots;
+    int64_t evicted_slots;   /* the same for evictions; one that the vertex's own visit finds out reads no more */
     int64_t changed;         /* vertices whose core moved by one */
     int64_t changed_slots;
     int64_t waves;           /* discovery + eviction waves */
@@ -149,8 +150,8 @@ typedef struct cm_stats {
     int64_t barriers;        /* barriers executed by the maintenance launches */
     int64_t grid_iterations; /* iterations run grid-wide (the rest ran in one block) */
     int64_t phase_ns[7];     /* device time per phase: claim, check, apply, discover, evict, commit, fix-up;
-                                for cm_recompute_cores / cm_create: level scans, sub-waves, chunk phases
-                                of the peel (the rest zero) */
+                                for cm_recompute_cores / cm_create: the peel's levels, and the sub-waves
+                                of work that its blocks share (the rest zero) */
     int64_t reserved[4];
 } cm_stats;
 

@@ -24,7 +24,6 @@
 using namespace cm;
 
 static thread_local std::string g_create_err = "no error";
-constexpr int kGridThreadsHost = 384;   // threads per block of the grid-mode kernels (kGridThreads)
 
 struct cm_graph {
     cm_options opt;
@@ -390,7 +389,7 @@ static int ensure_batch(cm_graph* h, long long k) {
 // with all blocks), so the bound follows the graph too, one thread per 32
 // list entries.
 static void persistent_geometry(cm_graph* h, long long work, int* blocks, int* threads) {
-    const int t = kGridThreadsHost;
+    const int t = kGridThreads;
     int occ = maintain_blocks_per_sm(t);
     if (occ < 1) occ = 1;
     int bps = h->opt.blocks_per_sm > 0 ? (h->opt.blocks_per_sm < occ ? h->opt.blocks_per_sm : occ) : occ;
@@ -1495,12 +1494,12 @@ static MaintainParams step_params(const cm_step* s, int op, int* blocks, int* th
     p.hub_len = c.hub_slots > 0 ? (c.hub_slots < 128 ? 128 : c.hub_slots) : c.hub_slots < 0 ? 0 : 1024;
     p.block_len = op == CM_OP_INSERT ? (c.block_slots >= 32 ? c.block_slots : 4096) : h->block_len_del;
     p.claim_max = c.task_claim >= 1 && c.task_claim <= 8 ? c.task_claim : 1;
-    int occ = maintain_blocks_per_sm(kGridThreadsHost);
+    int occ = maintain_blocks_per_sm(kGridThreads);
     if (occ < 1) occ = 1;
     int bps = c.blocks_per_sm > 0 && c.blocks_per_sm < occ ? c.blocks_per_sm : occ;
     int sms = h->opt.max_sms > 0 && h->opt.max_sms < h->num_sms ? h->opt.max_sms : h->num_sms;
     *blocks = sms * bps;
-    *threads = kGridThreadsHost;
+    *threads = kGridThreads;
     p.expect = (uint32_t)*blocks;
     return p;
 }

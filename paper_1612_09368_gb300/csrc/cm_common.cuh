@@ -143,8 +143,7 @@ struct __align__(128) Ctl {
     long long bad_index;           // smallest invalid input position
     unsigned long long gather_n;   // gathered incident edges (vertex deletion)
     unsigned long long reused;     // buckets of deleted keys that the inserted ones took
-    int min_deg;                   // peel: smallest remaining degree
-    int defer;                     // captured step: skip its remaining kernels (1 pool short, 2 error)
+    int defer;                     // skip the call's or step's remaining kernels (1 pool short, 2 error)
     unsigned long long passes;     // captured step: launch pairs of the current phase
     // grid-mode task queue of the current search (reset before each search)
     alignas(128) unsigned long long task_head;  // next slot a warp claims

@@ -68,13 +68,12 @@
 namespace cm {
 
 constexpr int kBlockThreads = 512;    // single-block mode
-// Grid mode, per block, two blocks per SM: 80 registers a thread.  The search
+// kGridThreads (cm_launch.h), with two blocks per SM: 80 registers a thread.  The search
 // needs about 90; at 64 (512 threads) the spills, which are written through to
 // L2, cost more than the warps gain.  512 / 448 / 384 / 320 threads, one pass
 // of inserts and deletes: R-MAT scale 20 with 10^4 edges 3.4 / 3.2 / 3.0 / 3.1
 // ms, Erdos-Renyi 2*10^6 with 10^4 4.2 / 4.1 / 4.0 / 3.9 ms, R-MAT scale 24
 // with 10^3 degree-proportional - / 10.3 / 9.7 / 10.4 ms.
-constexpr int kGridThreads = 384;
 static_assert(kGridThreads / 32 == kGridWarps, "one search buffer per grid-mode warp");
 constexpr int kMaxBig = 64;
 constexpr int kBlockLenSingle = 256;   // single-block mode: the block scans lists from this size
@@ -732,7 +731,8 @@ static const void* maintain_kernel(int mode, int op) {
 }
 
 // Resident blocks per SM of the grid-mode kernels (both operations).  Their
-// search buffers exceed the default 48 KB of shared memory per block.
+// search buffers take 40 KB of shared memory per block; the attribute is only
+// needed past 48 KB.
 int maintain_blocks_per_sm(int threads) {
     int least = 0;
     for (int op = 0; op < 2; op++) {

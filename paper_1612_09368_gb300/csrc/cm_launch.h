@@ -14,6 +14,8 @@ struct __align__(16) BSet {
     uint32_t pad;
 };
 
+constexpr int kGridThreads = 384;   // threads per block of the grid-mode maintenance kernels (cm_iterate.cu: why)
+
 // Parameters of a maintenance launch; where the call stands (remaining
 // edges, epoch, mode) lives in Ctl::rs.
 struct MaintainParams {
